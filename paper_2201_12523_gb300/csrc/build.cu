@@ -5,10 +5,13 @@
 //                 range check of every coordinate;
 //   radix sort    stable LSD sort of (linear index, input position), 8-bit
 //                 digits; per-tile digit counts, one exclusive scan, and a
-//                 stable per-tile scatter ranked with __match_any_sync;
-//   k_reencode    per stored nonzero: in-block key = concatenated per-mode
-//                 low fields, mode 0 lowest (Fig. 6b), value and input
-//                 position gathered, packed block key = bits above the line;
+//                 stable per-tile scatter ranked with warp votes;
+//   k_respread    per stored nonzero: the sorted linear index's bits moved to
+//                 the in-block key = concatenated per-mode low fields, mode 0
+//                 lowest (Fig. 6b), and to the packed block key = bits above
+//                 the line; value gathered by input position. Linear indices
+//                 of more than 64 bits take k_reencode, which forms the same
+//                 from the coordinates;
 //   runs/blocks   block boundaries where the block key changes (Section 4.2),
 //                 compacted on the device, split at the cap on the host.
 #include <algorithm>
@@ -77,20 +80,46 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 
 struct LinArgs {
     int N;
-    int B;
     uint32_t dims_m1[MAXN];  // I_n - 1
     int bits[MAXN];
+    int table[MAXN];         // first byte table of mode n
+    int ntables;
     uint8_t keypos[MAXN][32];
 };
 
 // ---------------------------------------------------------------------------
-// ALTO key of every nonzero; lo = key bits 0..63, hi = bits 64..127
+// ALTO key of every nonzero; lo = key bits 0..63, hi = bits 64..127 (WIDE).
+//
+// The key is an OR over the bytes of the coordinates: a shared-memory table
+// per byte holds where its 8 bits go. Moving the bits one by one took 670 warp
+// instructions per 32 nonzeros and 2.7 ms for 100M nonzeros of three modes (54
+// bits), bound by the integer pipes; the tables take 0.53 ms,
+// bound by their shared-memory reads.
 // ---------------------------------------------------------------------------
-__global__ void k_linearize(const uint32_t *__restrict__ coords, int64_t nnz, const LinArgs a,
-                            uint64_t *__restrict__ lo, uint64_t *__restrict__ hi, uint32_t *__restrict__ idx,
-                            unsigned long long *__restrict__ first_bad) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < nnz;
-         j += (int64_t)gridDim.x * blockDim.x) {
+template <bool WIDE>
+__global__ void __launch_bounds__(256) k_linearize(const uint32_t *__restrict__ coords, int64_t nnz, const LinArgs a,
+                                                   uint64_t *__restrict__ lo, uint64_t *__restrict__ hi,
+                                                   unsigned long long *__restrict__ first_bad) {
+    extern __shared__ uint64_t tab[];  // [ntables][256] low words, then high words (WIDE)
+    for (int i = threadIdx.x; i < a.ntables * 256; i += blockDim.x) {
+        const int t = i >> 8, v = i & 255;
+        int n = 0;
+        while (n + 1 < a.N && t >= a.table[n + 1]) ++n;
+        const int first = (t - a.table[n]) * 8;
+        uint64_t l = 0, h = 0;
+        for (int k = 0; k < 8 && first + k < a.bits[n]; ++k) {
+            const uint64_t bit = (v >> k) & 1;
+            const int p = a.keypos[n][first + k];
+            if (p < 64)
+                l |= bit << p;
+            else
+                h |= bit << (p - 64);
+        }
+        tab[i] = l;
+        if (WIDE) tab[a.ntables * 256 + i] = h;
+    }
+    __syncthreads();
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < nnz; j += (int64_t)gridDim.x * blockDim.x) {
         uint64_t l = 0, h = 0;
         bool bad = false;
 #pragma unroll
@@ -98,20 +127,20 @@ __global__ void k_linearize(const uint32_t *__restrict__ coords, int64_t nnz, co
             if (n < a.N) {
                 const uint32_t c = coords[j * a.N + n];
                 bad |= c > a.dims_m1[n];
-                for (int lev = 0; lev < a.bits[n]; ++lev) {
-                    const uint64_t bit = (c >> lev) & 1u;
-                    const int p = a.keypos[n][lev];
-                    if (p < 64)
-                        l |= bit << p;
-                    else
-                        h |= bit << (p - 64);
+                const uint64_t *t = tab + a.table[n] * 256;
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    if (b * 8 < a.bits[n]) {
+                        const uint32_t v = b * 256 + ((c >> (b * 8)) & 255u);
+                        l |= t[v];
+                        if (WIDE) h |= t[a.ntables * 256 + v];
+                    }
                 }
             }
         }
         if (bad) atomicMin(first_bad, (unsigned long long)j);
         lo[j] = l;
-        if (hi) hi[j] = h;
-        idx[j] = (uint32_t)j;
+        if (WIDE) hi[j] = h;
     }
 }
 
@@ -215,6 +244,21 @@ constexpr int kRsWarps = kRsThreads / 32;
 constexpr int kRsRounds = 16;
 constexpr int kRsTile = kRsThreads * kRsRounds;  // 4096 items
 
+// Lanes with the same 8-bit digit, among the valid ones: one vote per digit bit.
+// __match_any_sync takes a time that grows with the number of distinct values:
+// with it the count over 100M keys took 0.27-0.62 ms by digit and the scatter
+// 0.64-0.83, with the votes 0.31 and 0.63-0.70.
+__device__ __forceinline__ unsigned same_digit(uint32_t dg, bool valid) {
+    unsigned peers = __ballot_sync(kFull, valid);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool bit = (dg >> b) & 1u;
+        const unsigned v = __ballot_sync(kFull, bit);
+        peers &= bit ? v : ~v;
+    }
+    return peers;
+}
+
 template <typename K>
 __global__ void __launch_bounds__(kRsThreads) k_rs_count(const K *__restrict__ keys, int64_t n, int shift,
                                                          uint32_t *__restrict__ counts, int64_t ntiles) {
@@ -223,54 +267,60 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_count(const K *__restrict__ k
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * kRsTile;
     const int lane = threadIdx.x & 31;
+#pragma unroll 8
     for (int r = 0; r < kRsRounds; ++r) {
         const int64_t p = base + (int64_t)r * kRsThreads + threadIdx.x;
         const bool valid = p < n;
-        const uint32_t dg = valid ? (uint32_t)((keys[p] >> shift) & 0xFFu) : 256u;
-        const unsigned peers = __match_any_sync(kFull, dg);
+        const uint32_t dg = valid ? (uint32_t)((keys[p] >> shift) & 0xFFu) : 0u;
+        const unsigned peers = same_digit(dg, valid);
         if (valid && lane == __ffs(peers) - 1) atomicAdd(&hist[dg], (uint32_t)__popc(peers));
     }
     __syncthreads();
     counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = hist[threadIdx.x];
 }
 
+// Bound by latency, so by the warps in flight: with every item's key, value
+// and rank in registers (143 of them) one CTA fitted an SM, and a pass over
+// 100M (8 + 4)-byte items took 1.9 ms; with values read only where they are
+// staged and two ranks per register three CTAs fit: 0.64-0.83 ms by digit, and
+// 0.63-0.70 with the votes of same_digit().
 template <typename K>
-__global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const K *__restrict__ kin, const uint32_t *__restrict__ vin,
-                                                           K *__restrict__ kout, uint32_t *__restrict__ vout,
-                                                           int64_t n, int shift, const uint32_t *__restrict__ offs,
-                                                           int64_t ntiles) {
+__global__ void __launch_bounds__(kRsThreads, 3) k_rs_scatter(const K *__restrict__ kin,
+                                                              const uint32_t *__restrict__ vin, K *__restrict__ kout,
+                                                              uint32_t *__restrict__ vout, int64_t n, int shift,
+                                                              const uint32_t *__restrict__ offs, int64_t ntiles) {
     extern __shared__ __align__(16) unsigned char smem[];
     K *sk = reinterpret_cast<K *>(smem);
     uint32_t *sv = reinterpret_cast<uint32_t *>(sk + kRsTile);
     uint32_t *whist = sv + kRsTile;            // [kRsWarps][256]
     uint32_t *tbase = whist + kRsWarps * 256;  // [256]
-    uint32_t *tmp = tbase + 256;               // [32]
+    uint32_t *gbase = tbase + 256;             // [256] global offset of the digit's run minus tbase
+    uint32_t *tmp = gbase + 256;               // [32]
 
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * kRsTile;
+    const int tile_n = n - base < kRsTile ? (int)(n - base) : kRsTile;
+    // warp w ranks items [w*512, w*512+512) of the tile, 32 at a time, in order
+    const int it0 = w * (kRsTile / kRsWarps) + lane;
+    K kr[kRsRounds];
+#pragma unroll
+    for (int r = 0; r < kRsRounds; ++r) kr[r] = it0 + r * 32 < tile_n ? kin[base + it0 + r * 32] : (K)0;
     for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) whist[i] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRsTile;
-    const int64_t tile_n64 = n - base < kRsTile ? n - base : kRsTile;
-    const int tile_n = (int)tile_n64;
 
-    K kr[kRsRounds];
-    uint32_t vr[kRsRounds];
-    uint32_t rr[kRsRounds];
-    // warp w ranks items [w*512, w*512+512) of the tile, 32 at a time, in order
+    uint32_t rr[kRsRounds / 2];  // ranks, two per word
 #pragma unroll
     for (int r = 0; r < kRsRounds; ++r) {
-        const int it = w * (kRsTile / kRsWarps) + r * 32 + lane;
-        const bool valid = it < tile_n;
-        kr[r] = valid ? kin[base + it] : (K)0;
-        vr[r] = valid ? vin[base + it] : 0u;
-        const uint32_t dg = valid ? (uint32_t)((kr[r] >> shift) & 0xFFu) : 256u;
-        const unsigned peers = __match_any_sync(kFull, dg);
+        const bool valid = it0 + r * 32 < tile_n;
+        const uint32_t dg = (uint32_t)((kr[r] >> shift) & 0xFFu);
+        const unsigned peers = same_digit(dg, valid);
         const int leader = __ffs(peers) - 1;
-        const uint32_t prev = valid ? whist[w * 256 + (dg & 0xFFu)] : 0u;
+        const uint32_t prev = whist[w * 256 + dg];
         __syncwarp();
         if (valid && lane == leader) whist[w * 256 + dg] = prev + (uint32_t)__popc(peers);
         __syncwarp();
-        rr[r] = prev + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+        const uint32_t rank = prev + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+        rr[r / 2] = (r & 1) ? rr[r / 2] | (rank << 16) : rank;
     }
     __syncthreads();
     // per digit: exclusive over warps, and the tile total
@@ -285,26 +335,27 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const K *__restrict__
         }
         total_d = run;
     }
+    const uint32_t goff = offs[(int64_t)threadIdx.x * ntiles + blockIdx.x];
     __syncthreads();
     uint32_t all;
     const uint32_t excl = block_exclusive_scan(total_d, tmp, all);
     tbase[threadIdx.x] = excl;
+    gbase[threadIdx.x] = goff - excl;  // positions are below 2^32; the difference wraps
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < kRsRounds; ++r) {
-        const int it = w * (kRsTile / kRsWarps) + r * 32 + lane;
+        const int it = it0 + r * 32;
         if (it < tile_n) {
             const uint32_t dg = (uint32_t)((kr[r] >> shift) & 0xFFu);
-            const uint32_t lp = tbase[dg] + whist[w * 256 + dg] + rr[r];
+            const uint32_t lp = tbase[dg] + whist[w * 256 + dg] + ((rr[r / 2] >> ((r & 1) * 16)) & 0xFFFFu);
             sk[lp] = kr[r];
-            sv[lp] = vr[r];
+            sv[lp] = vin ? vin[base + it] : (uint32_t)(base + it);
         }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < tile_n; i += kRsThreads) {
         const K k = sk[i];
-        const uint32_t dg = (uint32_t)((k >> shift) & 0xFFu);
-        const int64_t gp = (int64_t)offs[(int64_t)dg * ntiles + blockIdx.x] + (i - (int64_t)tbase[dg]);
+        const uint32_t gp = gbase[(uint32_t)((k >> shift) & 0xFFu)] + (uint32_t)i;
         kout[gp] = k;
         vout[gp] = sv[i];
     }
@@ -312,38 +363,44 @@ __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const K *__restrict__
 
 template <typename K>
 size_t rs_scatter_smem() {
-    return sizeof(K) * kRsTile + sizeof(uint32_t) * kRsTile + sizeof(uint32_t) * (kRsWarps * 256 + 256 + 32);
+    return sizeof(K) * kRsTile + sizeof(uint32_t) * kRsTile + sizeof(uint32_t) * (kRsWarps * 256 + 512 + 32);
 }
 
-// Sorts (keys, vals) by key bits [0, nbits); result ends in (keys, vals).
+int rs_passes(int nbits) { return (nbits + 7) / 8; }
+
+// Sorts (key, value) pairs by key bits [0, nbits), at least one, in
+// rs_passes(nbits) passes that alternate between the two pairs of buffers; the
+// result ends in (keys, vals). The keys are read from `keys` after an even
+// number of passes' worth, else from `kalt`: key_source() says which. With
+// vals_in NULL the values are the positions 0..n-1. `counts` is scratch of
+// 256 * ceil(n / kRsTile) words.
 template <typename K>
-cudaError_t radix_sort_pairs(K *keys, uint32_t *vals, K *kalt, uint32_t *valt, int64_t n, int nbits,
-                             cudaStream_t s) {
-    if (n <= 1 || nbits <= 0) return cudaSuccess;
+K *key_source(K *keys, K *kalt, int nbits) {
+    return (rs_passes(nbits) & 1) ? kalt : keys;
+}
+template <typename K>
+cudaError_t radix_sort_pairs(K *keys, uint32_t *vals, K *kalt, uint32_t *valt, const uint32_t *vals_in, int64_t n,
+                             int nbits, uint32_t *counts, cudaStream_t s) {
     const int64_t ntiles = (n + kRsTile - 1) / kRsTile;
-    uint32_t *counts = nullptr;
-    cudaError_t e = cudaMallocAsync(&counts, sizeof(uint32_t) * 256 * ntiles, s);
-    if (e != cudaSuccess) return e;
     const size_t shm = rs_scatter_smem<K>();
-    e = cudaFuncSetAttribute(k_rs_scatter<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-    K *ki = keys, *ko = kalt;
-    uint32_t *vi = vals, *vo = valt;
-    for (int shift = 0; shift < nbits && e == cudaSuccess; shift += 8) {
-        k_rs_count<K><<<(unsigned)ntiles, kRsThreads, 0, s>>>(ki, n, shift, counts, ntiles);
+    cudaError_t e = cudaFuncSetAttribute(k_rs_scatter<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    const int passes = rs_passes(nbits);
+    K *ki = key_source(keys, kalt, nbits);
+    const uint32_t *vi = vals_in;
+    for (int i = 0; i < passes && e == cudaSuccess; ++i) {
+        const bool to_main = ((passes - i) & 1) != 0;
+        K *ko = to_main ? keys : kalt;
+        uint32_t *vo = to_main ? vals : valt;
+        k_rs_count<K><<<(unsigned)ntiles, kRsThreads, 0, s>>>(ki, n, 8 * i, counts, ntiles);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = scan_exclusive(counts, 256 * ntiles, s);
         if (e == cudaSuccess) {
-            k_rs_scatter<K><<<(unsigned)ntiles, kRsThreads, shm, s>>>(ki, vi, ko, vo, n, shift, counts, ntiles);
+            k_rs_scatter<K><<<(unsigned)ntiles, kRsThreads, shm, s>>>(ki, vi, ko, vo, n, 8 * i, counts, ntiles);
             e = cudaGetLastError();
         }
-        std::swap(ki, ko);
-        std::swap(vi, vo);
+        ki = ko;
+        vi = vo;
     }
-    if (e == cudaSuccess && ki != keys) {
-        e = cudaMemcpyAsync(keys, ki, sizeof(K) * n, cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(vals, vi, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s);
-    }
-    cudaFreeAsync(counts, s);
     return e;
 }
 
@@ -384,6 +441,71 @@ __global__ void k_reencode(const uint32_t *__restrict__ coords, const float *__r
         skeys[j] = key;
         svals[j] = vals ? vals[p] : 0.f;  // no float32 values: a float64 store gathers its own
         if (a.has_blocks) bkey[j] = bk;
+    }
+}
+
+// Where the bits of a linear index of at most 64 bits go: byte b's tables are
+// key[b][256], and, for stores with block-key bits, bkey[b][256].
+struct SpreadArgs {
+    int nbytes;
+    int has_blocks;
+    uint8_t to[64];  // destination of linear-index bit p: key bit, or 64 + block-key bit
+};
+
+// In-block key, block key and value of every stored nonzero from the sorted
+// linear indices (`lin` may be `skeys`). Reading the coordinates by input
+// position instead (k_reencode) took 4.4 ms for 100M nonzeros of three modes,
+// a random 12-byte read each; this takes 2.1, most of it the values'.
+template <bool BLOCKS>
+__global__ void __launch_bounds__(256) k_respread(const uint64_t *lin, const float *__restrict__ vals,
+                                                  const uint32_t *__restrict__ perm, int64_t nnz, const SpreadArgs a,
+                                                  uint64_t *skeys, float *__restrict__ svals,
+                                                  uint64_t *__restrict__ bkey) {
+    extern __shared__ uint64_t tab[];
+    for (int i = threadIdx.x; i < a.nbytes * 256; i += blockDim.x) {
+        uint64_t k = 0, b = 0;
+        for (int j = 0; j < 8; ++j) {
+            const int to = a.to[((i >> 8) * 8 + j) & 63];
+            const uint64_t bit = (i >> j) & 1;
+            if (to < 64)
+                k |= bit << to;
+            else if (to < 128)
+                b |= bit << (to - 64);
+        }
+        tab[i] = k;
+        if (BLOCKS) tab[a.nbytes * 256 + i] = b;
+    }
+    __syncthreads();
+    // four elements per thread in flight: the values are random reads
+    constexpr int U = 4;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t j0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j0 < nnz; j0 += U * step) {
+        uint64_t l[U];
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t j = j0 + u * step;
+            l[u] = j < nnz ? lin[j] : 0ull;
+            v[u] = j < nnz && vals ? vals[perm[j]] : 0.f;  // no float32 values: a float64 store gathers its own
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t j = j0 + u * step;
+            uint64_t key = 0, bk = 0;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                if (b < a.nbytes) {
+                    const int t = b * 256 + (int)((l[u] >> (8 * b)) & 255u);
+                    key |= tab[t];
+                    if (BLOCKS) bk |= tab[a.nbytes * 256 + t];
+                }
+            }
+            if (j < nnz) {
+                skeys[j] = key;
+                svals[j] = v[u];
+                if (BLOCKS) bkey[j] = bk;
+            }
+        }
     }
 }
 
@@ -430,7 +552,18 @@ __global__ void k_tile_block(const int64_t *__restrict__ bstart, int64_t nblocks
 // `stride`-th 32-nonzero tile (all tiles when stride is 1), one warp per
 // sampled tile. The counts only rank rows for on-chip accumulation, so a
 // sample of tens of millions of nonzeros is enough to find the heavy rows.
+// Short modes (SMEM) count in shared memory first: a 2048-row mode of 100M
+// nonzeros took 1.6 ms with all atomics on the same few rows in L2, 0.27 so.
+constexpr int kHistRows = 8192;
+
+template <bool SMEM>
 __global__ void k_histogram(const StoreView sv, int mode, int64_t stride, uint32_t *__restrict__ counts) {
+    extern __shared__ uint32_t local[];
+    const int nrows = (int)sv.dims[mode];  // used where SMEM: at most kHistRows
+    if (SMEM) {
+        for (int i = threadIdx.x; i < nrows; i += blockDim.x) local[i] = 0;
+        __syncthreads();
+    }
     const int64_t ntiles = (sv.end - sv.begin + 31) >> 5;
     const int64_t nsamp = (ntiles + stride - 1) / stride;
     const int lane = threadIdx.x & 31;
@@ -453,17 +586,19 @@ __global__ void k_histogram(const StoreView sv, int mode, int64_t stride, uint32
         const unsigned lanes = __ballot_sync(0xFFFFFFFFu, live);
         if (live) {
             const unsigned peers = __match_any_sync(lanes, row);
-            if (lane == __ffs(peers) - 1) atomicAdd(&counts[row], (uint32_t)__popc(peers));
+            if (lane == __ffs(peers) - 1) atomicAdd(SMEM ? &local[row] : &counts[row], (uint32_t)__popc(peers));
         }
+    }
+    if (SMEM) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < nrows; i += blockDim.x)
+            if (local[i]) atomicAdd(&counts[i], local[i]);
     }
 }
 
-__global__ void k_pack_count_row(const uint32_t *__restrict__ counts, int64_t I, uint32_t *__restrict__ key,
-                                 uint32_t *__restrict__ row) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < I; i += (int64_t)gridDim.x * blockDim.x) {
+__global__ void k_complement(const uint32_t *__restrict__ counts, int64_t I, uint32_t *__restrict__ key) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < I; i += (int64_t)gridDim.x * blockDim.x)
         key[i] = ~counts[i];  // ascending sort of ~count = descending count
-        row[i] = (uint32_t)i;
-    }
 }
 
 unsigned grid_for(int64_t n, int threads) {
@@ -474,6 +609,13 @@ unsigned grid_for(int64_t n, int threads) {
     return (unsigned)g;
 }
 
+// Grid of a kernel whose CTAs begin by filling byte tables: few enough CTAs
+// that each has many elements to amortize that over.
+unsigned table_grid(int64_t n) {
+    const int64_t need = (n + 2047) / 2048;
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sm_count() * 8));
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -481,8 +623,10 @@ cudaError_t build_store(const Layout &L, const uint32_t *coords, const float *va
                         BuildOut &out, cudaStream_t s, std::string &why) {
     cudaError_t e = cudaSuccess;
     const int64_t npad = ((nnz + 31) / 32) * 32 + 32;
-    uint64_t *lo = nullptr, *lo2 = nullptr, *hi = nullptr, *hi2 = nullptr, *bkey = nullptr;
-    uint32_t *idx = nullptr, *idx2 = nullptr;
+    const int64_t nbits = std::min(std::max(L.B, 1), 64);  // sorted low bits (a length-1 shape has none: one pass)
+    uint64_t *lo = nullptr, *hi = nullptr, *hi2 = nullptr, *bkey = nullptr;
+    uint64_t *d_rkeys = nullptr;
+    uint32_t *idx = nullptr, *idx2 = nullptr, *counts = nullptr, *flags = nullptr;
     unsigned long long *d_bad = nullptr;
     const bool wide = L.B > 64;
     const bool has_blocks = L.B > L.line;
@@ -491,33 +635,47 @@ cudaError_t build_store(const Layout &L, const uint32_t *coords, const float *va
         e = (x);                    \
         if (e != cudaSuccess) goto done; \
     } while (0)
+    // The store's own arrays serve as one half of the sort's buffers (keys and
+    // positions; the values' array, filled last, holds the other positions);
+    // only the second key buffer is scratch. Plain cudaMalloc: memory of the
+    // default stream-ordered pool goes back to the device at the next
+    // synchronization, which costs 2.3 ms per GB and call against 0.5.
     TRY(cudaMalloc(&out.keys, sizeof(uint64_t) * npad));
     TRY(cudaMalloc(&out.vals, sizeof(float) * npad));
     TRY(cudaMalloc(&out.perm, sizeof(uint32_t) * (nnz > 0 ? nnz : 1)));
-    TRY(cudaMemsetAsync(out.keys, 0, sizeof(uint64_t) * npad, s));
-    TRY(cudaMemsetAsync(out.vals, 0, sizeof(float) * npad, s));
+    TRY(cudaMemsetAsync(out.keys + nnz, 0, sizeof(uint64_t) * (npad - nnz), s));
+    TRY(cudaMemsetAsync(out.vals + nnz, 0, sizeof(float) * (npad - nnz), s));
     if (nnz > 0) {
-        TRY(cudaMallocAsync(&lo, sizeof(uint64_t) * nnz, s));
-        TRY(cudaMallocAsync(&lo2, sizeof(uint64_t) * nnz, s));
-        TRY(cudaMallocAsync(&idx2, sizeof(uint32_t) * nnz, s));
+        const int64_t ntiles = (nnz + kRsTile - 1) / kRsTile;
+        TRY(cudaMalloc(&lo, sizeof(uint64_t) * nnz));
+        TRY(cudaMallocAsync(&counts, sizeof(uint32_t) * 256 * ntiles, s));
         TRY(cudaMallocAsync(&d_bad, sizeof(unsigned long long), s));
         TRY(cudaMemsetAsync(d_bad, 0xFF, sizeof(unsigned long long), s));
         idx = out.perm;
+        idx2 = reinterpret_cast<uint32_t *>(out.vals);
         if (wide) {
-            TRY(cudaMallocAsync(&hi, sizeof(uint64_t) * nnz, s));
-            TRY(cudaMallocAsync(&hi2, sizeof(uint64_t) * nnz, s));
+            TRY(cudaMalloc(&hi, sizeof(uint64_t) * nnz));
+            TRY(cudaMalloc(&hi2, sizeof(uint64_t) * nnz));
         }
         {
             LinArgs a;
             memset(&a, 0, sizeof(a));
             a.N = L.N;
-            a.B = L.B;
             for (int n = 0; n < L.N; ++n) {
                 a.dims_m1[n] = (uint32_t)(L.dims[n] - 1);
                 a.bits[n] = L.bits[n];
+                a.table[n] = a.ntables;
+                a.ntables += (L.bits[n] + 7) / 8;
                 memcpy(a.keypos[n], L.keypos[n], 32);
             }
-            k_linearize<<<grid_for(nnz, 256), 256, 0, s>>>(coords, nnz, a, lo, hi, idx, d_bad);
+            uint64_t *src = key_source(out.keys, lo, (int)nbits);
+            const size_t shm = (size_t)a.ntables * 256 * sizeof(uint64_t) * (wide ? 2 : 1);
+            if (wide) {
+                TRY(cudaFuncSetAttribute(k_linearize<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+                k_linearize<true><<<table_grid(nnz), 256, shm, s>>>(coords, nnz, a, src, hi, d_bad);
+            } else {
+                k_linearize<false><<<table_grid(nnz), 256, shm, s>>>(coords, nnz, a, src, nullptr, d_bad);
+            }
             TRY(cudaGetLastError());
         }
         {
@@ -531,13 +689,23 @@ cudaError_t build_store(const Layout &L, const uint32_t *coords, const float *va
             }
         }
         // sort by the low word, then (stably) by the high word
-        TRY(radix_sort_pairs<uint64_t>(lo, idx, lo2, idx2, nnz, std::min(L.B, 64), s));
+        TRY(radix_sort_pairs<uint64_t>(out.keys, idx, lo, idx2, nullptr, nnz, (int)nbits, counts, s));
         if (wide) {
             k_gather_u64<<<grid_for(nnz, 256), 256, 0, s>>>(hi, idx, nnz, hi2);
             TRY(cudaGetLastError());
-            TRY(radix_sort_pairs<uint64_t>(hi2, idx, hi, idx2, nnz, L.B - 64, s));
+            // an odd number of passes reads from its second key buffer and
+            // ends in its first: hi2 is the source either way; the positions
+            // start in idx, so they may not be the first pass's output
+            const bool odd = (rs_passes(L.B - 64) & 1) != 0;
+            if (odd) {
+                TRY(cudaMemcpyAsync(idx2, idx, sizeof(uint32_t) * nnz, cudaMemcpyDeviceToDevice, s));
+                TRY(radix_sort_pairs<uint64_t>(hi, idx, hi2, idx2, idx2, nnz, L.B - 64, counts, s));
+            } else {
+                TRY(radix_sort_pairs<uint64_t>(hi2, idx, hi, idx2, idx, nnz, L.B - 64, counts, s));
+            }
         }
-        {
+        if (has_blocks) TRY(cudaMalloc(&bkey, sizeof(uint64_t) * nnz));
+        if (wide) {
             EncArgs a;
             memset(&a, 0, sizeof(a));
             a.N = L.N;
@@ -548,17 +716,31 @@ cudaError_t build_store(const Layout &L, const uint32_t *coords, const float *va
                 a.width[n] = L.width[n];
                 a.boff[n] = L.boff[n];
             }
-            if (has_blocks) TRY(cudaMallocAsync(&bkey, sizeof(uint64_t) * nnz, s));
             k_reencode<<<grid_for(nnz, 256), 256, 0, s>>>(coords, vals, idx, nnz, a, out.keys, out.vals, bkey);
-            TRY(cudaGetLastError());
+        } else {
+            SpreadArgs a;
+            memset(&a, 0, sizeof(a));
+            a.nbytes = (L.B + 7) / 8;
+            a.has_blocks = has_blocks ? 1 : 0;
+            memset(a.to, 0xFF, sizeof(a.to));  // no such bit
+            for (int n = 0; n < L.N; ++n)
+                for (int l = 0; l < L.bits[n]; ++l)
+                    a.to[L.keypos[n][l]] =
+                        (uint8_t)(l < L.width[n] ? L.shift[n] + l : 64 + L.boff[n] + (l - L.width[n]));
+            const size_t shm = (size_t)a.nbytes * 256 * sizeof(uint64_t) * (has_blocks ? 2 : 1);
+            if (has_blocks)
+                k_respread<true><<<table_grid(nnz), 256, shm, s>>>(out.keys, vals, idx, nnz, a, out.keys, out.vals, bkey);
+            else
+                k_respread<false><<<table_grid(nnz), 256, shm, s>>>(out.keys, vals, idx, nnz, a, out.keys, out.vals, bkey);
         }
+        TRY(cudaGetLastError());
     }
     // block runs
     {
         std::vector<int64_t> run_start;
         std::vector<uint64_t> run_key;
         if (nnz > 0 && has_blocks) {
-            uint32_t *flags = idx2;  // reuse
+            TRY(cudaMallocAsync(&flags, sizeof(uint32_t) * nnz, s));
             k_run_flags<<<grid_for(nnz, 256), 256, 0, s>>>(bkey, nnz, flags);
             TRY(cudaGetLastError());
             uint32_t last_flag = 0;
@@ -568,8 +750,8 @@ cudaError_t build_store(const Layout &L, const uint32_t *coords, const float *va
             TRY(cudaMemcpyAsync(&last_scan, flags + nnz - 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
             TRY(cudaStreamSynchronize(s));
             const int64_t nruns = (int64_t)last_scan + last_flag;
-            int64_t *d_starts = reinterpret_cast<int64_t *>(lo2);  // reuse: nruns <= nnz
-            uint64_t *d_rkeys = lo;
+            int64_t *d_starts = reinterpret_cast<int64_t *>(lo);  // reuse: nruns <= nnz
+            TRY(cudaMallocAsync(&d_rkeys, sizeof(uint64_t) * nruns, s));
             k_run_compact<<<grid_for(nnz, 256), 256, 0, s>>>(bkey, flags, nnz, d_starts, d_rkeys);
             TRY(cudaGetLastError());
             run_start.resize(nruns);
@@ -602,14 +784,18 @@ cudaError_t build_store(const Layout &L, const uint32_t *coords, const float *va
     }
 done:
 #undef TRY
-    if (lo) cudaFreeAsync(lo, s);
-    if (lo2) cudaFreeAsync(lo2, s);
-    if (hi) cudaFreeAsync(hi, s);
-    if (hi2) cudaFreeAsync(hi2, s);
-    if (idx2) cudaFreeAsync(idx2, s);
-    if (bkey) cudaFreeAsync(bkey, s);
+    if (counts) cudaFreeAsync(counts, s);
+    if (flags) cudaFreeAsync(flags, s);
+    if (d_rkeys) cudaFreeAsync(d_rkeys, s);
     if (d_bad) cudaFreeAsync(d_bad, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    {
+        const cudaError_t es = cudaStreamSynchronize(s);  // also before the scratch goes, whatever happened
+        if (e == cudaSuccess) e = es;
+    }
+    if (lo) cudaFree(lo);
+    if (hi) cudaFree(hi);
+    if (hi2) cudaFree(hi2);
+    if (bkey) cudaFree(bkey);
     return e;
 }
 
@@ -632,27 +818,31 @@ cudaError_t mode_histogram(const StoreView &sv, int mode, uint32_t *counts, cuda
     const int64_t ntiles = (sv.end - sv.begin + 31) / 32;
     const int64_t stride = std::max<int64_t>(1, ntiles >> 20);  // at most ~2^20 sampled tiles
     const int64_t nsamp = (ntiles + stride - 1) / stride;
-    k_histogram<<<grid_for(nsamp * 32, 256), 256, 0, s>>>(sv, mode, stride, counts);
+    if (sv.dims[mode] <= kHistRows)
+        k_histogram<true><<<grid_for(nsamp * 32, 256), 256, sizeof(uint32_t) * sv.dims[mode], s>>>(sv, mode, stride, counts);
+    else
+        k_histogram<false><<<grid_for(nsamp * 32, 256), 256, 0, s>>>(sv, mode, stride, counts);
     return cudaGetLastError();
 }
 
 cudaError_t top_rows(const uint32_t *counts, int64_t I, int k, uint32_t *rows_out, cudaStream_t s) {
-    uint32_t *key = nullptr, *row = nullptr, *key2 = nullptr, *row2 = nullptr;
+    uint32_t *key = nullptr, *row = nullptr, *key2 = nullptr, *row2 = nullptr, *tiles = nullptr;
+    const int64_t ntiles = (I + kRsTile - 1) / kRsTile;
     cudaError_t e = cudaMallocAsync(&key, sizeof(uint32_t) * I, s);
     if (e == cudaSuccess) e = cudaMallocAsync(&row, sizeof(uint32_t) * I, s);
     if (e == cudaSuccess) e = cudaMallocAsync(&key2, sizeof(uint32_t) * I, s);
     if (e == cudaSuccess) e = cudaMallocAsync(&row2, sizeof(uint32_t) * I, s);
+    if (e == cudaSuccess) e = cudaMallocAsync(&tiles, sizeof(uint32_t) * 256 * ntiles, s);
     if (e == cudaSuccess) {
-        k_pack_count_row<<<grid_for(I, 256), 256, 0, s>>>(counts, I, key, row);
+        static_assert(32 / 8 % 2 == 0, "an even number of passes reads from and ends in `key`");
+        k_complement<<<grid_for(I, 256), 256, 0, s>>>(counts, I, key);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = radix_sort_pairs<uint32_t>(key, row, key2, row2, I, 32, s);
+    if (e == cudaSuccess) e = radix_sort_pairs<uint32_t>(key, row, key2, row2, nullptr, I, 32, tiles, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(rows_out, row, sizeof(uint32_t) * std::min<int64_t>(k, I), cudaMemcpyDeviceToDevice, s);
-    if (key) cudaFreeAsync(key, s);
-    if (row) cudaFreeAsync(row, s);
-    if (key2) cudaFreeAsync(key2, s);
-    if (row2) cudaFreeAsync(row2, s);
+    for (uint32_t *b : {key, row, key2, row2, tiles})
+        if (b) cudaFreeAsync(b, s);
     return e;
 }
 
