@@ -20,7 +20,8 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libblco.so")
 SOURCES = ["api.cu", "build.cu", "mttkrp.cu", "mttkrp_f32.cu", "mttkrp_bf16.cu", "mttkrp_f16.cu", "mttkrp_fused.cu", "mttkrp_f64.cu",
-           "dense.cu"]
+           "tile_order.cu", "mttkrp_tiled_f32.cu", "mttkrp_tiled_bf16.cu", "mttkrp_tiled_f16.cu",
+           "mttkrp_tiled_f64.cu", "dense.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -46,6 +47,7 @@ def _stale(target: str, deps) -> bool:
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
     headers = [os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "mttkrp_kernels.cuh"),
+               os.path.join(CSRC, "mttkrp_tiled.cuh"), os.path.join(CSRC, "hot_rows.cuh"),
                os.path.join(INCLUDE, "blco.h")]
     objs, jobs = [], []
     for src in SOURCES:

@@ -31,6 +31,11 @@ int sm_count() {
 namespace {
 
 constexpr int64_t kDefaultCap = (int64_t)1 << 27;
+// Fewest nonzeros for which the order inside tiles is kept. Measured on one
+// MTTKRP (host call included; tile order against 32 at a time, R = 32): 300k
+// nonzeros 14-19 us against 19-24, 600k 18-25 against 25-41; at 64k a launch is
+// mostly latency either way (64 tiles).
+constexpr int64_t kOrderMinNnz = (int64_t)1 << 16;
 
 blco_status fail(blco_status st, const std::string &msg) {
     g_err = msg;
@@ -110,6 +115,9 @@ struct blco_tensor {
     // hot rows per mode
     uint32_t *d_hot[MAXN] = {};
     int hot_count[MAXN] = {};
+    // order inside tiles (resident stores; NULL: none)
+    void *d_order = nullptr;
+    TileOrder order;
     // streaming queues
     int64_t queue_nnz = 0;
     uint64_t *q_keys[8] = {};
@@ -208,6 +216,7 @@ void release(blco_tensor *h) {
     h->dfree(h->d_bbase, 0);
     h->dfree(h->d_tile_block, 0);
     for (int n = 0; n < MAXN; ++n) h->dfree(h->d_hot[n], 0);
+    h->dfree(h->d_order, 0);
     for (int q = 0; q < 8; ++q) {
         h->dfree(h->q_keys[q], 0);
         h->dfree(h->q_vals[q], 0);
@@ -444,6 +453,15 @@ HotRows hot_for(const blco_tensor *h, int mode, int R) {
     return hr;
 }
 
+// The most frequent rows of `mode`, for kernels that choose how many they hold.
+HotRows hot_all(const blco_tensor *h, int mode) {
+    HotRows hr;
+    hr.rows = h->d_hot[mode];
+    hr.count = h->hot_count[mode];
+    hr.dense = 0;
+    return hr;
+}
+
 // Device memory for n private output copies of `floats` each; false (and
 // no error left pending) when it cannot be had, e.g. under a device budget.
 bool copy_buffer(blco_tensor *h, size_t bytes, float **p) {
@@ -478,9 +496,11 @@ blco_status mttkrp_device(blco_tensor *h, int mode, const FactorSet &fs, blco_dt
     }
     cudaError_t e = timed(h, "zero", s, [&]() { return launch_zero(dst, n * oc.n, s); });
     if (e != cudaSuccess) return cuda_fail(e, "zero output");
+    const bool tiled = h->d_order && range_end < 0 && !(h->compensated && fdt != BLCO_F32);
     blco_status st = over_store(
         h, "mttkrp", vals_ext, s,
         [&](const StoreView &sv, cudaStream_t q) {
+            if (tiled) return launch_mttkrp_tiled(sv, h->order, fs, fdt, R, mode, hot_all(h, mode), dst, oc, q);
             return launch_mttkrp(sv, fs, fdt, R, mode, hot, dst, oc, h->compensated, q);
         },
         range_begin, range_end);
@@ -717,6 +737,24 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
     }
     h->building = false;
     if (h->budget > 0 && h->dev_bytes > h->budget) BAIL(fail(BLCO_ERR_OOM, "device budget exceeded"));
+    // The order inside tiles: for stores without a device budget (which is the
+    // caller's to divide) that have it in a quarter of the free memory. A store
+    // without it is served by the kernels that order 32 nonzeros at a time.
+    if (!h->streamed && h->budget == 0 && tile_order_supported(h->L) && nnz >= kOrderMinNnz) {
+        const size_t ob = tile_order_bytes(nnz, N, no_vals);
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && ob <= free_b / 4 &&
+            h->dalloc(&h->d_order, ob) == cudaSuccess) {
+            h->order = tile_order_view(h->d_order, nnz, N, no_vals);
+            HotRows hot[MAXN];
+            for (int n = 0; n < N; ++n) hot[n] = hot_all(h, n);
+            e = build_tile_order(h->view(), h->L, hot, h->order, s);
+            if (e != cudaSuccess) BAIL(cuda_fail(e, "tile order"));
+        } else {
+            cudaGetLastError();
+            h->d_order = nullptr;
+        }
+    }
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) BAIL(cuda_fail(e, "construction"));
 cleanup:
@@ -850,7 +888,10 @@ blco_status blco_mttkrp_f64(blco_handle h, int mode, const double *const *factor
     if (e != cudaSuccess) return cuda_fail(e, "zero output");
     if (h->nnz > 0) {
         StoreView sv = h->view();
-        e = timed(h, "mttkrp_f64", s, [&]() { return launch_mttkrp_f64(sv, fs, R, mode, hot, o, s); });
+        e = timed(h, "mttkrp_f64", s, [&]() {
+            if (h->d_order) return launch_mttkrp_tiled_f64(sv, h->order, fs, R, mode, hot_all(h, mode), o, s);
+            return launch_mttkrp_f64(sv, fs, R, mode, hot, o, s);
+        });
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     }
     if (host_out) {

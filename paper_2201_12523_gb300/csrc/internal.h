@@ -14,6 +14,8 @@ namespace blco {
 
 constexpr int MAXN = BLCO_MAX_MODES;
 constexpr uint32_t kNoRow = 0xFFFFFFFFu;  // never a valid index: I_n < 2^32
+constexpr int kTile = 1024;     // store positions of one tile of the tile order
+constexpr int kOrderCold = 63;  // tile order: place of a row that is not among the 63 hottest
 
 // ---------------------------------------------------------------------------
 // Layout of the store (Sections 4.1-4.2), computed on the host at build time.
@@ -55,6 +57,13 @@ struct StoreView {
 
 struct FactorSet {
     const void *ptr[MAXN];
+};
+
+// The order inside tiles of kTile store positions (tile_order.cu), per mode.
+struct TileOrder {
+    uint16_t *rank[MAXN] = {};   // per store position: rank inside its tile | place of its row among the hottest << 10
+    uint32_t *ends[MAXN] = {};   // bit per rank: last nonzero of a run of equal target rows
+    uint32_t *fends[MAXN] = {};  // bit per rank: last nonzero of a fiber (equal target and partner rows); float64
 };
 
 // Hot output rows of one mode (accumulated in shared memory).
@@ -101,6 +110,24 @@ bool rank_supported(int R);
 bool fused_supported(const StoreView &sv, int R);
 cudaError_t launch_mttkrp_fused(const StoreView &sv, const FactorSet &fs, blco_dtype fdt, int R, const HotRows *hot,
                                 float *const *outs, cudaStream_t s);
+// tile_order.cu
+int order_partner(const int64_t *dims, int N, int mode);
+bool tile_order_supported(const Layout &L);  // at least two modes, of at most 2^31 rows each
+size_t tile_order_bytes(int64_t nnz, int N, bool fibers);
+TileOrder tile_order_view(void *buf, int64_t nnz, int N, bool fibers);
+cudaError_t build_tile_order(const StoreView &sv, const Layout &L, const HotRows *hot, const TileOrder &to,
+                             cudaStream_t s);
+// mttkrp_tiled_*.cu: the MTTKRP of a whole store with its tile order
+cudaError_t launch_mttkrp_tiled(const StoreView &sv, const TileOrder &to, const FactorSet &fs, blco_dtype fdt, int R,
+                                int mode, const HotRows &hot, float *out, const OutCopies &oc, cudaStream_t s);
+cudaError_t launch_mttkrp_tiled_f32(const StoreView &sv, const TileOrder &to, const FactorSet &fs, int R, int mode,
+                                    const HotRows &hot, float *out, const OutCopies &oc, cudaStream_t s);
+cudaError_t launch_mttkrp_tiled_bf16(const StoreView &sv, const TileOrder &to, const FactorSet &fs, int R, int mode,
+                                     const HotRows &hot, float *out, const OutCopies &oc, cudaStream_t s);
+cudaError_t launch_mttkrp_tiled_f16(const StoreView &sv, const TileOrder &to, const FactorSet &fs, int R, int mode,
+                                    const HotRows &hot, float *out, const OutCopies &oc, cudaStream_t s);
+cudaError_t launch_mttkrp_tiled_f64(const StoreView &sv, const TileOrder &to, const double *const *factors, int R,
+                                    int mode, const HotRows &hot, double *out, cudaStream_t s);
 // mttkrp_f64.cu: float64 values, factors and output
 cudaError_t launch_mttkrp_f64(const StoreView &sv, const double *const *factors, int R, int mode, const HotRows &hot,
                               double *out, cudaStream_t s);

@@ -19,6 +19,16 @@ cudaError_t launch_mttkrp(const StoreView &sv, const FactorSet &fs, blco_dtype f
     return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_mttkrp_tiled(const StoreView &sv, const TileOrder &to, const FactorSet &fs, blco_dtype fdt, int R,
+                                int mode, const HotRows &hot, float *out, const OutCopies &oc, cudaStream_t s) {
+    switch (fdt) {
+        case BLCO_F32: return launch_mttkrp_tiled_f32(sv, to, fs, R, mode, hot, out, oc, s);
+        case BLCO_BF16: return launch_mttkrp_tiled_bf16(sv, to, fs, R, mode, hot, out, oc, s);
+        case BLCO_F16: return launch_mttkrp_tiled_f16(sv, to, fs, R, mode, hot, out, oc, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
 // A short mode's output receives most of a launch's reductions on few rows;
 // private copies spread them. Measured on GB300: at R = 64 (16 rows per warp
 // on chip, 16 vector reductions per nonzero) a 1024-row mode ran 18% faster

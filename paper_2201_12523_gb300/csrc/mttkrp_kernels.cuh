@@ -40,6 +40,7 @@
 
 #include <cstring>
 
+#include "hot_rows.cuh"
 #include "internal.h"
 
 // Kernels and launchers are templates over the factor type; each of
@@ -191,7 +192,9 @@ struct Chunk<__nv_bfloat16> {
     static constexpr int PAIRS = 2;
     static constexpr int BYTES = 8;
     __device__ __forceinline__ static void load(const void *addr, f2 *f) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(addr));
+        widen(__ldg(reinterpret_cast<const uint2 *>(addr)), f);
+    }
+    __device__ __forceinline__ static void widen(const uint2 v, f2 *f) {
         f[0] = bf16x2_to_f2(v.x);
         f[1] = bf16x2_to_f2(v.y);
     }
@@ -202,7 +205,9 @@ struct Chunk<__half> {
     static constexpr int PAIRS = 2;
     static constexpr int BYTES = 8;
     __device__ __forceinline__ static void load(const void *addr, f2 *f) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(addr));
+        widen(__ldg(reinterpret_cast<const uint2 *>(addr)), f);
+    }
+    __device__ __forceinline__ static void widen(const uint2 v, f2 *f) {
         const uint32_t w[2] = {v.x, v.y};
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -249,10 +254,6 @@ __device__ __forceinline__ uint32_t block_of(const KParams &p, int64_t pos) {
     uint32_t b = __ldg(p.tile_block + (pos >> 5));
     while (pos >= __ldg(p.bstart + b + 1)) ++b;
     return b;
-}
-
-__device__ __forceinline__ uint32_t hot_hash(uint32_t row, int log2n) {
-    return log2n > 0 ? (row * 0x9E3779B1u) >> (32 - log2n) : 0u;
 }
 
 // Number of gathered modes: NG > 0 fixed at compile time, NG == 0 runtime.

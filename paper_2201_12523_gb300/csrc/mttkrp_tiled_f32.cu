@@ -1,0 +1,11 @@
+// Tile-order MTTKRP kernels for float factors.
+#include "mttkrp_tiled.cuh"
+
+namespace blco {
+
+cudaError_t launch_mttkrp_tiled_f32(const StoreView &sv, const TileOrder &to, const FactorSet &fs, int R, int mode,
+                                    const HotRows &hot, float *out, const OutCopies &oc, cudaStream_t s) {
+    return tiled_as<float>(sv, to, fs, R, mode, hot, out, oc, s);
+}
+
+}  // namespace blco
