@@ -1,6 +1,6 @@
 // Dense helpers around the sparse kernels: output zeroing, float32 ->
 // 16-bit factor conversion, and the FP64 pieces of CP-ALS (Algorithm 1):
-// Grams, the Hadamard product of Grams, its Cholesky (or eigen
+// Grams, the Hadamard product of Grams, its inverse (or eigen
 // pseudo-inverse) solve, column normalization and the fit.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -60,14 +60,21 @@ __device__ __forceinline__ float to_f<__half>(__half v) { return __half2float(v)
 // shared memory in float64, and CTAs meet in float64 atomics (both halves of
 // an off-diagonal block). This keeps the FP64 pipe, which is a small fraction
 // of the FP32 rate on this GPU, off the O(I R^2) part of the work.
+//
+// Bound by the ten float32 operations per product. CTAs are as wide as whole
+// thread groups need (at most kGramThreads): with 256 threads, R = 64 left one
+// group of 136 threads and the other 120 idle, and 2^20 rows took 1.30 ms; two
+// groups in 288 threads take 1.09.
 constexpr int kGramRows = 32;  // rows staged in shared memory per step
-constexpr int kGramThreads = 256;
+constexpr int kGramThreads = 288;
 
 struct GramShape {
     int R4;      // R rounded up to 4 (padding columns are zero)
     int B;       // 4 x 4 blocks per side
     int nblk;    // blocks in the upper triangle
-    int groups;  // thread groups per CTA that split the rows (nblk < 256)
+    int ny;      // parts of the blocks, one per blockIdx.y
+    int per_y;   // blocks of a part
+    int groups;  // thread groups per CTA that split the rows
 };
 
 __host__ __device__ inline GramShape gram_shape(int R) {
@@ -75,7 +82,9 @@ __host__ __device__ inline GramShape gram_shape(int R) {
     g.R4 = (R + 3) & ~3;
     g.B = g.R4 / 4;
     g.nblk = g.B * (g.B + 1) / 2;
-    g.groups = g.nblk >= kGramThreads ? 1 : kGramThreads / g.nblk;
+    g.ny = (g.nblk + kGramThreads - 1) / kGramThreads;
+    g.per_y = (g.nblk + g.ny - 1) / g.ny;
+    g.groups = kGramThreads / g.per_y;
     return g;
 }
 
@@ -85,23 +94,49 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kGramThreads) k_gram(const T *__restrict__ A, int64_t I, int R, int64_t rows_per_cta,
+// One more term x * y of a Dot2 sum (hi, lo).
+__device__ __forceinline__ void dot2_add(float x, float y, float &hi, float &lo) {
+    const float p = __fmul_rn(x, y);
+    const float e = __fmaf_rn(x, y, -p);  // x*y == p + e exactly
+    float sum, err;
+    two_sum(hi, p, sum, err);
+    hi = sum;
+    lo = __fadd_rn(lo, __fadd_rn(err, e));
+}
+
+// Column scales from the columns' sums of squares: lambda = sqrt, 1 / lambda
+// (1 for a zero column).
+__device__ __forceinline__ float inv_norm(double colsq, double *lambda) {
+    const double l = sqrt(colsq);
+    *lambda = l;
+    return l > 0.0 ? (float)(1.0 / l) : 1.f;
+}
+
+// With SCALE (float factors, one part of blocks), A's columns are first divided
+// by their norms, in place, and the Gram is that of the scaled A; CTA 0 writes
+// lambda. Scaling here instead of in a pass of its own saves that pass's read
+// and write (0.15 ms at 2^20 x 64).
+template <typename T, bool SCALE>
+__global__ void __launch_bounds__(kGramThreads, 3) k_gram(const T *A, T *A_out, int64_t I, int R, int64_t rows_per_cta,
+                                                       const double *__restrict__ colsq, double *__restrict__ lambda,
                                                        double *__restrict__ G) {
     extern __shared__ __align__(16) unsigned char smem[];
     const GramShape sh = gram_shape(R);
     float *tile = reinterpret_cast<float *>(smem);                       // kGramRows x R4
-    double *red = reinterpret_cast<double *>(tile + kGramRows * sh.R4);  // groups x nblk x 16
+    double *red = reinterpret_cast<double *>(tile + kGramRows * sh.R4);  // groups x per_y x 16
+    __shared__ float inv[SCALE ? 64 : 1];
     const int tid = threadIdx.x;
-    int blk, grp;
-    if (sh.groups > 1) {
-        blk = tid % sh.nblk;
-        grp = tid / sh.nblk;
-    } else {
-        blk = blockIdx.y * kGramThreads + tid;
-        grp = 0;
+    if (SCALE) {
+        if (tid < R) {
+            double l;
+            inv[tid] = inv_norm(colsq[tid], &l);
+            if (blockIdx.x == 0) lambda[tid] = l;
+        }
     }
-    const bool active = blk < sh.nblk && grp < sh.groups;
+    const int grp = tid / sh.per_y;
+    const int lbl = tid % sh.per_y;  // block inside the part
+    const int blk = blockIdx.y * sh.per_y + lbl;
+    const bool active = grp < sh.groups && blk < sh.nblk && (!SCALE || G);
     int br = 0, rem = active ? blk : 0;  // upper-triangle block -> (br, bc)
     while (rem >= sh.B - br) {
         rem -= sh.B - br;
@@ -113,12 +148,38 @@ __global__ void __launch_bounds__(kGramThreads) k_gram(const T *__restrict__ A, 
     for (int k = 0; k < 16; ++k) hi[k] = lo[k] = 0.f;
     const int64_t r0 = (int64_t)blockIdx.x * rows_per_cta;
     const int64_t r1 = r0 + rows_per_cta < I ? r0 + rows_per_cta : I;
+    // rows of whole 16-byte words (8 bytes of 16-bit factors) move four at a time
+    const bool vec = sizeof(T) == 4 && R == sh.R4 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
     for (int64_t b0 = r0; b0 < r1; b0 += kGramRows) {
         const int nr = (int)((r1 - b0) < kGramRows ? (r1 - b0) : kGramRows);
         __syncthreads();
-        for (int i = tid; i < kGramRows * sh.R4; i += kGramThreads) {
-            const int row = i / sh.R4, col = i % sh.R4;
-            tile[i] = (row < nr && col < R) ? to_f<T>(A[(b0 + row) * R + col]) : 0.f;
+        if (vec) {
+            const float4 *src = reinterpret_cast<const float4 *>(A + b0 * R);
+            for (int i = tid; i < kGramRows * sh.B; i += blockDim.x) {
+                float4 v = i < nr * sh.B ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (SCALE && i < nr * sh.B) {
+                    const int c = i % sh.B * 4;
+                    v.x *= inv[c];
+                    v.y *= inv[c + 1];
+                    v.z *= inv[c + 2];
+                    v.w *= inv[c + 3];
+                    reinterpret_cast<float4 *>(A_out + b0 * R)[i] = v;
+                }
+                reinterpret_cast<float4 *>(tile)[i] = v;
+            }
+        } else {
+            for (int i = tid; i < kGramRows * sh.R4; i += blockDim.x) {
+                const int row = i / sh.R4, col = i % sh.R4;
+                float v = 0.f;
+                if (row < nr && col < R) {
+                    v = to_f<T>(A[(b0 + row) * R + col]);
+                    if constexpr (SCALE) {
+                        v *= inv[col];
+                        A_out[(b0 + row) * R + col] = v;
+                    }
+                }
+                tile[i] = v;
+            }
         }
         __syncthreads();
         if (!active) continue;
@@ -129,32 +190,21 @@ __global__ void __launch_bounds__(kGramThreads) k_gram(const T *__restrict__ A, 
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const float p = __fmul_rn(xa[u], ya[v]);
-                    const float e = __fmaf_rn(xa[u], ya[v], -p);  // x*y == p + e exactly
-                    float sum, err;
-                    two_sum(hi[u * 4 + v], p, sum, err);
-                    hi[u * 4 + v] = sum;
-                    lo[u * 4 + v] = __fadd_rn(lo[u * 4 + v], __fadd_rn(err, e));
-                }
+                for (int v = 0; v < 4; ++v) dot2_add(xa[u], ya[v], hi[u * 4 + v], lo[u * 4 + v]);
         }
     }
-    // sum the thread groups of this CTA in float64, then one atomic per
-    // entry. Shared slots are indexed by the block's local index: with thread
-    // groups the block itself, else the thread (blockIdx.y picks the range).
-    const int nloc = sh.groups > 1 ? sh.nblk : kGramThreads;  // local blocks per group
-    const int lbl = sh.groups > 1 ? blk : tid;
+    if (SCALE && !G) return;
+    // sum the thread groups of this CTA in float64, then one atomic per entry
     if (active)
 #pragma unroll
-        for (int k = 0; k < 16; ++k) red[(grp * nloc + lbl) * 16 + k] = (double)hi[k] + (double)lo[k];
+        for (int k = 0; k < 16; ++k) red[(grp * sh.per_y + lbl) * 16 + k] = (double)hi[k] + (double)lo[k];
     __syncthreads();
-    const int nact = sh.groups > 1 ? sh.nblk : min(kGramThreads, sh.nblk - (int)blockIdx.y * kGramThreads);
-    for (int i = tid; i < nact * 16; i += kGramThreads) {
+    const int nact = min(sh.per_y, sh.nblk - (int)blockIdx.y * sh.per_y);
+    for (int i = tid; i < nact * 16; i += blockDim.x) {
         const int lb = i / 16, k = i % 16;
         double v = 0.0;
-        for (int g2 = 0; g2 < sh.groups; ++g2) v += red[(g2 * nloc + lb) * 16 + k];
-        const int gb = sh.groups > 1 ? lb : (int)blockIdx.y * kGramThreads + lb;
-        int rr = 0, rm = gb;
+        for (int g2 = 0; g2 < sh.groups; ++g2) v += red[(g2 * sh.per_y + lb) * 16 + k];
+        int rr = 0, rm = (int)blockIdx.y * sh.per_y + lb;
         while (rm >= sh.B - rr) {
             rm -= sh.B - rr;
             ++rr;
@@ -175,25 +225,43 @@ struct GramPtrs {
 };
 
 // -------------------------------------------------------------------------
-// one CTA: V = Hadamard of Grams (k != mode); W = V^{-1} by Cholesky, or the
-// eigen pseudo-inverse (cyclic Jacobi) when V is not positive definite.
-// Output W as float32 (the apply step) and info.
+// one CTA: V = Hadamard of Grams (k != mode); W = V^{-1}, or the eigen
+// pseudo-inverse (cyclic Jacobi) when V is not positive definite. Output W as
+// float32 (the apply step) and info; zeroes the column sums of squares that
+// the apply step adds to.
+//
+// The inverse is Gauss-Jordan elimination on the symmetric matrix (the sweep
+// operator, J. H. Goodnight, The American Statistician 33(3), 1979): its pivots
+// are the squares of Cholesky's, so positive definiteness is decided as a
+// Cholesky factorization decides it. The lower triangle stays in registers
+// (R (R + 1) / 2 entries over 256 threads) and a step passes only its pivot
+// column through shared memory. Bound by the one SM's FP64 pipe at R = 64
+// (R^2 / 2 multiply-adds per step) and by the step's chain (reciprocal, two
+// barriers) at R = 32: Cholesky with one thread per column of the inverse took
+// 376 us at R = 64 and 129 us at R = 32, this 154 and 62.
 // -------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_solve_small(const GramPtrs gp, int N, int mode, int R,
-                                                     float *__restrict__ Wf, int32_t *__restrict__ info) {
+constexpr int kSolveThreads = 256;
+constexpr int kSolveMaxRank = 64;
+constexpr int kSolveSlots = (kSolveMaxRank * (kSolveMaxRank + 1) / 2 + kSolveThreads - 1) / kSolveThreads;
+
+__global__ void __launch_bounds__(kSolveThreads) k_solve_small(const GramPtrs gp, int N, int mode, int R,
+                                                               float *__restrict__ Wf, double *__restrict__ colsq,
+                                                               int32_t *__restrict__ info) {
     extern __shared__ __align__(16) unsigned char smem[];
-    double *V = reinterpret_cast<double *>(smem);  // R x R: V, then W (or Jacobi vectors)
+    double *V = reinterpret_cast<double *>(smem);  // R x R: V, then the Jacobi vectors
     double *L = V + R * R;                           // R x R work
-    __shared__ int ok;
     const int tid = threadIdx.x;
-    for (int p = tid; p < R * R; p += blockDim.x) {
+    if (tid < R) colsq[tid] = 0.0;
+    for (int p = tid; p < R * R; p += kSolveThreads) {
         double v = 1.0;
         for (int k = 0; k < N; ++k)
             if (k != mode) v *= gp.g[k][p];
         V[p] = v;
-        L[p] = v;
     }
-    __shared__ double pd_tol;
+    __shared__ double pd_tol, rcp;
+    __shared__ double col[kSolveMaxRank], colr[kSolveMaxRank];
+    __shared__ int ok;
+    __syncthreads();
     if (tid == 0) {
         ok = 1;
         // smallest pivot accepted as positive: R * eps * max_i V_ii; at or
@@ -203,45 +271,59 @@ __global__ void __launch_bounds__(256) k_solve_small(const GramPtrs gp, int N, i
         for (int i = 0; i < R; ++i) m = fmax(m, V[i * R + i]);
         pd_tol = (double)R * 2.220446049250313e-16 * m;
     }
-    __syncthreads();
-    // Cholesky, right-looking, in L (lower triangle)
+    // entry (row, column) of the lower triangle in slot q of this thread
+    const int ntri = R * (R + 1) / 2;
+    double x[kSolveSlots];
+    int ri[kSolveSlots], ci[kSolveSlots];
+#pragma unroll
+    for (int q = 0; q < kSolveSlots; ++q) {
+        const int t = tid + q * kSolveThreads;
+        int i = 0, rest = t;
+        while (rest > i) {
+            rest -= i + 1;
+            ++i;
+        }
+        ri[q] = t < ntri ? i : -1;
+        ci[q] = t < ntri ? rest : -1;
+        x[q] = t < ntri ? V[i * R + rest] : 0.0;
+    }
     for (int j = 0; j < R; ++j) {
-        if (tid == 0) {
-            const double d = L[j * R + j];
-            if (!(d > pd_tol)) ok = 0;
-            L[j * R + j] = d > 0.0 ? sqrt(d) : 1.0;
+        // the pivot's row and column
+#pragma unroll
+        for (int q = 0; q < kSolveSlots; ++q) {
+            if (ci[q] == j) col[ri[q]] = x[q];
+            else if (ri[q] == j) col[ci[q]] = x[q];
+            if (ri[q] == j && ci[q] == j) rcp = 1.0 / x[q];
+        }
+        __syncthreads();
+        if (tid < R) {
+            colr[tid] = col[tid] * rcp;
+            if (tid == j && !(col[j] > pd_tol)) ok = 0;
         }
         __syncthreads();
         if (!ok) break;
-        const double djj = L[j * R + j];
-        for (int i = j + 1 + tid; i < R; i += blockDim.x) L[i * R + j] /= djj;
-        __syncthreads();
-        for (int p = tid; p < (R - j - 1) * (R - j - 1); p += blockDim.x) {
-            const int i = j + 1 + p / (R - j - 1), k = j + 1 + p % (R - j - 1);
-            if (k <= i) L[i * R + k] -= L[i * R + j] * L[k * R + j];
+#pragma unroll
+        for (int q = 0; q < kSolveSlots; ++q) {
+            if (ri[q] < 0) continue;
+            if (ri[q] == j)
+                x[q] = ci[q] == j ? -rcp : colr[ci[q]];
+            else if (ci[q] == j)
+                x[q] = colr[ri[q]];
+            else
+                x[q] = fma(-colr[ri[q]], col[ci[q]], x[q]);
         }
         __syncthreads();
     }
     if (ok) {
-        // W = L^{-T} L^{-1}, one column per thread, in place in V[:, c]
-        __syncthreads();
-        for (int c = tid; c < R; c += blockDim.x) {
-            for (int i = 0; i < R; ++i) {  // forward: L x = e_c
-                double sum = (i == c) ? 1.0 : 0.0;
-                for (int k = 0; k < i; ++k) sum -= L[i * R + k] * V[k * R + c];
-                V[i * R + c] = sum / L[i * R + i];
-            }
-            for (int i = R - 1; i >= 0; --i) {  // back: L^T w = x
-                double sum = V[i * R + c];
-                for (int k = i + 1; k < R; ++k) sum -= L[k * R + i] * V[k * R + c];
-                V[i * R + c] = sum / L[i * R + i];
-            }
+#pragma unroll
+        for (int q = 0; q < kSolveSlots; ++q) {
+            if (ri[q] < 0) continue;
+            Wf[ri[q] * R + ci[q]] = Wf[ci[q] * R + ri[q]] = (float)-x[q];
         }
-        __syncthreads();
-        for (int p = tid; p < R * R; p += blockDim.x) Wf[p] = (float)V[p];
         if (tid == 0) *info = 0;
         return;
     }
+    __syncthreads();
     // ---- eigen pseudo-inverse: cyclic Jacobi rotations on L := V, Q := I
     double *Q = V;
     for (int p = tid; p < R * R; p += blockDim.x) {
@@ -337,100 +419,183 @@ __global__ void __launch_bounds__(256) k_solve_small(const GramPtrs gp, int N, i
     if (tid == 0) *info = 1;
 }
 
-// A = M W (float32, W in shared memory), one warp per row.
-__global__ void __launch_bounds__(256) k_apply(const float *__restrict__ M, int64_t I, int R,
-                                               const float *__restrict__ Wg, float *__restrict__ A) {
+// A = M W (float32) and the columns' sums of squares (Dot2, float64 between
+// threads and CTAs). A thread computes 4 rows x 4 columns of a tile staged in
+// shared memory, summing over k in increasing order with one FMA per term; A
+// may be M. G, if not NULL, is zeroed for the Gram that follows.
+//
+// Bound by the float32 FMAs at R = 64 (2 I R^2), by HBM at small R. One warp
+// per row with two shared loads per FMA took 0.95 ms at 2^20 x 64 and a
+// float64 pass for the sums of squares 0.25; together 0.27 here.
+constexpr int kApplyThreads = 256;
+
+struct ApplyShape {
+    int R4;      // R rounded up to 4
+    int cg, rg;  // column groups of 4, row groups
+    int rows;    // rows of a tile
+    int stride;  // floats per staged row: R4 + 4, so that neighbouring row groups hit different banks
+};
+__host__ __device__ inline ApplyShape apply_shape(int R) {
+    ApplyShape s;
+    s.R4 = (R + 3) & ~3;
+    s.cg = s.R4 / 4;
+    s.rg = kApplyThreads / s.cg;
+    s.rows = 4 * s.rg;
+    s.stride = s.R4 + 4;
+    return s;
+}
+inline size_t apply_smem(int R) {
+    const ApplyShape s = apply_shape(R);
+    const size_t stage = sizeof(float) * ((size_t)s.R4 * s.R4 + (size_t)s.rows * s.stride);
+    return std::max(stage, sizeof(double) * 4 * kApplyThreads);
+}
+
+__global__ void __launch_bounds__(kApplyThreads) k_apply(const float *M, int64_t I, int R,
+                                                         const float *__restrict__ Wg, float *A,
+                                                         double *__restrict__ colsq, double *__restrict__ G) {
     extern __shared__ __align__(16) unsigned char smem[];
-    float *W = reinterpret_cast<float *>(smem);
-    float *rowbuf = W + R * R;  // 8 warps x R
-    for (int p = threadIdx.x; p < R * R; p += blockDim.x) W[p] = Wg[p];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    float *rb = rowbuf + w * R;
-    for (int64_t i = (int64_t)blockIdx.x * 8 + w; i < I; i += (int64_t)gridDim.x * 8) {
-        for (int k = lane; k < R; k += 32) rb[k] = M[i * R + k];
-        __syncwarp();
-        for (int cidx = lane; cidx < R; cidx += 32) {
-            float s = 0.f;
-            for (int k = 0; k < R; ++k) s = fmaf(rb[k], W[k * R + cidx], s);
-            A[i * R + cidx] = s;
+    const ApplyShape sh = apply_shape(R);
+    float *W = reinterpret_cast<float *>(smem);  // R4 x R4, zero beyond R
+    float *Ms = W + sh.R4 * sh.R4;               // rows x stride, zero beyond R
+    const int tid = threadIdx.x;
+    const int c = tid % sh.cg * 4, rg = tid / sh.cg;
+    if (G && blockIdx.x == 0)
+        for (int p = tid; p < R * R; p += kApplyThreads) G[p] = 0.0;
+    for (int p = tid; p < sh.R4 * sh.R4; p += kApplyThreads) {
+        const int k = p / sh.R4, n = p % sh.R4;
+        W[p] = k < R && n < R ? Wg[k * R + n] : 0.f;
+    }
+    const bool vec = R == sh.R4 && ((reinterpret_cast<uintptr_t>(M) | reinterpret_cast<uintptr_t>(A)) & 15) == 0;
+    float hi[4], lo[4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) hi[n] = lo[n] = 0.f;
+    const int64_t ntiles = (I + sh.rows - 1) / sh.rows;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int64_t i0 = t * sh.rows;
+        const int nr = I - i0 < sh.rows ? (int)(I - i0) : sh.rows;
+        __syncthreads();
+        if (vec) {
+            const float4 *src = reinterpret_cast<const float4 *>(M + i0 * R);
+            for (int p = tid; p < nr * sh.cg; p += kApplyThreads)
+                *reinterpret_cast<float4 *>(Ms + p / sh.cg * sh.stride + p % sh.cg * 4) = src[p];
+        } else {
+            for (int p = tid; p < nr * sh.R4; p += kApplyThreads) {
+                const int r = p / sh.R4, k = p % sh.R4;
+                Ms[r * sh.stride + k] = k < R ? M[(i0 + r) * R + k] : 0.f;
+            }
         }
-        __syncwarp();
+        __syncthreads();
+        if (rg >= sh.rg) continue;
+        float acc[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int n = 0; n < 4; ++n) acc[a][n] = 0.f;
+        const float *mrow = Ms + rg * sh.stride;  // rows rg + a * sh.rg
+        for (int k = 0; k < sh.R4; k += 4) {
+            float m[4][4], w[4][4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+                *reinterpret_cast<float4 *>(m[a]) =
+                    *reinterpret_cast<const float4 *>(mrow + a * sh.rg * sh.stride + k);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+                *reinterpret_cast<float4 *>(w[kk]) = *reinterpret_cast<const float4 *>(W + (k + kk) * sh.R4 + c);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) acc[a][n] = fmaf(m[a][kk], w[kk][n], acc[a][n]);
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int r = rg + a * sh.rg;
+            if (r >= nr) continue;
+            float *dst = A + (i0 + r) * R + c;
+            if (vec) {
+                *reinterpret_cast<float4 *>(dst) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+            } else {
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+                    if (c + n < R) dst[n] = acc[a][n];
+            }
+#pragma unroll
+            for (int n = 0; n < 4; ++n) dot2_add(acc[a][n], acc[a][n], hi[n], lo[n]);
+        }
+    }
+    __syncthreads();
+    double *red = reinterpret_cast<double *>(smem);  // [rg][R4]
+    if (rg < sh.rg)
+#pragma unroll
+        for (int n = 0; n < 4; ++n) red[rg * sh.R4 + c + n] = (double)hi[n] + (double)lo[n];
+    __syncthreads();
+    if (tid < R) {
+        double v = 0.0;
+        for (int g = 0; g < sh.rg; ++g) v += red[g * sh.R4 + tid];
+        atomicAdd(&colsq[tid], v);
     }
 }
 
-// column sums of squares (float64) -> colsq[R] via atomics
-__global__ void __launch_bounds__(256) k_colsq(const float *__restrict__ A, int64_t I, int R, double *__restrict__ colsq) {
-    // thread handles column c = threadIdx.x % R for rows strided
-    const int lanes = 256 / R * R;  // threads used
-    if (threadIdx.x >= lanes) return;
-    const int c = threadIdx.x % R;
-    const int sub = threadIdx.x / R, nsub = 256 / R;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * nsub + sub; i < I; i += (int64_t)gridDim.x * nsub) {
-        const double v = A[i * R + c];
-        s += v * v;
-    }
-    atomicAdd(&colsq[c], s);
-}
-
-__global__ void k_sqrt_lambda(const double *__restrict__ colsq, int R, double *__restrict__ lambda,
-                              float *__restrict__ inv) {
-    const int c = threadIdx.x;
-    if (c < R) {
-        const double l = sqrt(colsq[c]);
-        lambda[c] = l;
-        inv[c] = l > 0.0 ? (float)(1.0 / l) : 1.f;
-    }
-}
-
-__global__ void k_scale_cols(float *__restrict__ A, int64_t I, int R, const float *__restrict__ inv) {
-    const int64_t n = I * R;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
-        A[p] *= inv[p % R];
-}
-
-// <M, A> per column (float64) -> acc[R]
+// <M, A> per column (Dot2, float64 between threads and CTAs) -> acc[R]
 __global__ void __launch_bounds__(256) k_coldot(const float *__restrict__ M, const float *__restrict__ A, int64_t I,
                                                 int R, double *__restrict__ acc) {
-    const int lanes = 256 / R * R;
-    if (threadIdx.x >= lanes) return;
-    const int c = threadIdx.x % R;
-    const int sub = threadIdx.x / R, nsub = 256 / R;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * nsub + sub; i < I; i += (int64_t)gridDim.x * nsub)
-        s += (double)M[i * R + c] * (double)A[i * R + c];
-    atomicAdd(&acc[c], s);
+    __shared__ double red[256];
+    const int nsub = 256 / R;
+    const int c = threadIdx.x % R, sub = threadIdx.x / R;
+    float hi = 0.f, lo = 0.f;
+    if (sub < nsub)
+        for (int64_t i = (int64_t)blockIdx.x * nsub + sub; i < I; i += (int64_t)gridDim.x * nsub)
+            dot2_add(M[i * R + c], A[i * R + c], hi, lo);
+    red[threadIdx.x] = (double)hi + (double)lo;
+    __syncthreads();
+    if (threadIdx.x < R) {
+        double v = 0.0;
+        for (int g = 0; g < nsub; ++g) v += red[g * R + threadIdx.x];
+        atomicAdd(&acc[threadIdx.x], v);
+    }
 }
 
-__global__ void k_fit_final(double normX2, const GramPtrs gp, int N, int R, const double *__restrict__ lambda,
-                            const double *__restrict__ dots, double *__restrict__ fit) {
-    __shared__ double part[256];
+__global__ void __launch_bounds__(256) k_fit_final(double normX2, const GramPtrs gp, int N, int R,
+                                                   const double *__restrict__ lambda,
+                                                   const double *__restrict__ dots, double *__restrict__ fit) {
+    __shared__ double part[8], inner[8];
     double s = 0.0;
-    for (int p = threadIdx.x; p < R * R; p += blockDim.x) {
+    for (int p = threadIdx.x; p < R * R; p += 256) {
         double v = 1.0;
         for (int k = 0; k < N; ++k) v *= gp.g[k][p];
         s += lambda[p / R] * v * lambda[p % R];
     }
-    part[threadIdx.x] = s;
+    double d = threadIdx.x < R ? lambda[threadIdx.x] * dots[threadIdx.x] : 0.0;
+    for (int o = 16; o >= 1; o >>= 1) {
+        s += __shfl_xor_sync(kFull, s, o);
+        d += __shfl_xor_sync(kFull, d, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        part[threadIdx.x >> 5] = s;
+        inner[threadIdx.x >> 5] = d;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double xh2 = 0.0;
-        for (int i = 0; i < (int)blockDim.x; ++i) xh2 += part[i];
-        double inner = 0.0;
-        for (int c = 0; c < R; ++c) inner += lambda[c] * dots[c];
-        double r2 = normX2 + xh2 - 2.0 * inner;
+        double xh2 = 0.0, in = 0.0;
+        for (int i = 0; i < 8; ++i) {
+            xh2 += part[i];
+            in += inner[i];
+        }
+        double r2 = normX2 + xh2 - 2.0 * in;
         if (r2 < 0.0) r2 = 0.0;
         *fit = 1.0 - sqrt(r2) / sqrt(normX2);
     }
 }
 
+// Dot2 per thread, float64 between threads: bound by the read of v (in float64
+// throughout, 8M values took 36 us; now 22).
 __global__ void __launch_bounds__(256) k_norm2(const float *__restrict__ v, int64_t n, double *__restrict__ out) {
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double x = v[i];
-        s += x * x;
-    }
+    float hi = 0.f, lo = 0.f;
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        dot2_add(v[i], v[i], hi, lo);
+    double s = (double)hi + (double)lo;
     for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
 }
@@ -482,80 +647,98 @@ cudaError_t launch_convert(const float *src, void *dst, blco_dtype dt, int64_t n
     return cudaGetLastError();
 }
 
+namespace {
+
+struct GramLaunch {
+    dim3 grid;
+    int threads;
+    size_t shm;
+    int64_t rows;
+};
+
+// three CTAs per SM in total (the register limit), each over a contiguous
+// range of rows
+GramLaunch gram_launch(int64_t I, int R) {
+    const GramShape sh = gram_shape(R);
+    const int64_t ctas_max = std::max<int64_t>(1, (int64_t)sm_count() * 3 / sh.ny);
+    GramLaunch g;
+    g.rows = (I + ctas_max - 1) / ctas_max;
+    g.rows = std::max<int64_t>(kGramRows, (g.rows + kGramRows - 1) / kGramRows * kGramRows);
+    g.threads = (sh.groups * sh.per_y + 31) / 32 * 32;
+    g.shm = sizeof(float) * kGramRows * sh.R4 + sizeof(double) * sh.groups * sh.per_y * 16;
+    g.grid = dim3((unsigned)((I + g.rows - 1) / g.rows), (unsigned)sh.ny);
+    return g;
+}
+
+template <typename T>
+cudaError_t run_gram(const void *A, int64_t I, int R, double *G, cudaStream_t s) {
+    const GramLaunch g = gram_launch(I, R);
+    cudaError_t e = cudaFuncSetAttribute(k_gram<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.shm);
+    if (e != cudaSuccess) return e;
+    k_gram<T, false><<<g.grid, g.threads, g.shm, s>>>(static_cast<const T *>(A), nullptr, I, R, g.rows, nullptr,
+                                                      nullptr, G);
+    return cudaGetLastError();
+}
+
+__global__ void k_zero_lambda(double *lambda, double *G, int R) {
+    for (int i = threadIdx.x; i < R; i += blockDim.x) lambda[i] = 0.0;
+    if (G)
+        for (int i = threadIdx.x; i < R * R; i += blockDim.x) G[i] = 0.0;
+}
+
+// The CP-ALS update of one factor with its scratch given: R x R floats, R doubles.
+cudaError_t run_update(const double *const *grams, int N, int mode, int R, const float *M, int64_t I, float *A,
+                       double *lambda, double *G_out, int32_t *info, float *Wf, double *colsq, cudaStream_t s) {
+    GramPtrs gp;
+    for (int k = 0; k < MAXN; ++k) gp.g[k] = k < N ? grams[k] : nullptr;
+    const size_t shm_solve = sizeof(double) * 2 * R * R;
+    cudaError_t e = cudaFuncSetAttribute(k_solve_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_solve);
+    if (e != cudaSuccess) return e;
+    k_solve_small<<<1, kSolveThreads, shm_solve, s>>>(gp, N, mode, R, Wf, colsq, info);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (I <= 0) {
+        k_zero_lambda<<<1, 256, 0, s>>>(lambda, G_out, R);
+        return cudaGetLastError();
+    }
+    const size_t shm = apply_smem(R);
+    e = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    if (e != cudaSuccess) return e;
+    const int64_t tiles = (I + apply_shape(R).rows - 1) / apply_shape(R).rows;
+    const int64_t ctas = std::min<int64_t>(tiles, (int64_t)sm_count() * 4);
+    k_apply<<<(unsigned)ctas, kApplyThreads, shm, s>>>(M, I, R, Wf, A, colsq, G_out);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const GramLaunch g = gram_launch(I, R);
+    e = cudaFuncSetAttribute(k_gram<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.shm);
+    if (e != cudaSuccess) return e;
+    k_gram<float, true><<<g.grid, g.threads, g.shm, s>>>(A, A, I, R, g.rows, colsq, lambda, G_out);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_gram(const void *A, blco_dtype fdt, int64_t I, int R, double *G, cudaStream_t s) {
     k_zero_d<<<1, 256, 0, s>>>(G, R * R);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || I <= 0) return e;
-    const GramShape sh = gram_shape(R);
-    const int ny = sh.groups > 1 ? 1 : (sh.nblk + kGramThreads - 1) / kGramThreads;
-    // three CTAs per SM in total (the register limit at 79 registers), each
-    // over a contiguous range of rows
-    const int64_t ctas_max = std::max<int64_t>(1, (int64_t)sm_count() * 3 / ny);
-    int64_t rows = (I + ctas_max - 1) / ctas_max;
-    rows = std::max<int64_t>(kGramRows, (rows + kGramRows - 1) / kGramRows * kGramRows);
-    const int64_t ctas = (I + rows - 1) / rows;
-    const size_t red_entries = (size_t)(sh.groups > 1 ? sh.groups * sh.nblk : kGramThreads) * 16;
-    const size_t shm = sizeof(float) * kGramRows * sh.R4 + sizeof(double) * red_entries;
-    const dim3 grid((unsigned)ctas, (unsigned)ny);
     switch (fdt) {
-        case BLCO_F32:
-            e = cudaFuncSetAttribute(k_gram<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-            if (e == cudaSuccess)
-                k_gram<float><<<grid, kGramThreads, shm, s>>>(static_cast<const float *>(A), I, R, rows, G);
-            break;
-        case BLCO_BF16:
-            e = cudaFuncSetAttribute(k_gram<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-            if (e == cudaSuccess)
-                k_gram<__nv_bfloat16><<<grid, kGramThreads, shm, s>>>(static_cast<const __nv_bfloat16 *>(A), I, R,
-                                                                        rows, G);
-            break;
-        case BLCO_F16:
-            e = cudaFuncSetAttribute(k_gram<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-            if (e == cudaSuccess)
-                k_gram<__half><<<grid, kGramThreads, shm, s>>>(static_cast<const __half *>(A), I, R, rows, G);
-            break;
+        case BLCO_F32: return run_gram<float>(A, I, R, G, s);
+        case BLCO_BF16: return run_gram<__nv_bfloat16>(A, I, R, G, s);
+        case BLCO_F16: return run_gram<__half>(A, I, R, G, s);
     }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_cpals_update(const double *const *grams, int N, int mode, int R, const float *M, int64_t I,
                                 float *A, double *lambda, double *G_out, int32_t *info, cudaStream_t s) {
-    GramPtrs gp;
-    for (int k = 0; k < MAXN; ++k) gp.g[k] = k < N ? grams[k] : nullptr;
-    float *Wf = nullptr;
-    double *colsq = nullptr;
-    float *inv = nullptr;
-    cudaError_t e = cudaMallocAsync(&Wf, sizeof(float) * R * R, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&colsq, sizeof(double) * R, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&inv, sizeof(float) * R, s);
-    if (e == cudaSuccess) {
-        const size_t shm = sizeof(double) * 2 * R * R;
-        e = cudaFuncSetAttribute(k_solve_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-        if (e == cudaSuccess) {
-            k_solve_small<<<1, 256, shm, s>>>(gp, N, mode, R, Wf, info);
-            e = cudaGetLastError();
-        }
-    }
-    if (e == cudaSuccess && I > 0) {
-        const size_t shm = sizeof(float) * (R * R + 8 * R);
-        e = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-        if (e == cudaSuccess) {
-            k_apply<<<grid_cap(I, 8), 256, shm, s>>>(M, I, R, Wf, A);
-            e = cudaGetLastError();
-        }
-    }
-    if (e == cudaSuccess) {
-        k_zero_d<<<1, 256, 0, s>>>(colsq, R);
-        if (I > 0) k_colsq<<<grid_cap(I, 256 / R), 256, 0, s>>>(A, I, R, colsq);
-        k_sqrt_lambda<<<1, 128, 0, s>>>(colsq, R, lambda, inv);
-        if (I > 0) k_scale_cols<<<grid_cap(I * R, 256), 256, 0, s>>>(A, I, R, inv);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess && G_out) e = launch_gram(A, BLCO_F32, I, R, G_out, s);
-    if (Wf) cudaFreeAsync(Wf, s);
-    if (colsq) cudaFreeAsync(colsq, s);
-    if (inv) cudaFreeAsync(inv, s);
+    unsigned char *buf = nullptr;
+    const size_t wf = (sizeof(float) * R * R + 255) / 256 * 256;
+    cudaError_t e = cudaMallocAsync(&buf, wf + sizeof(double) * R, s);
+    if (e != cudaSuccess) return e;
+    e = run_update(grams, N, mode, R, M, I, A, lambda, G_out, info, reinterpret_cast<float *>(buf),
+                   reinterpret_cast<double *>(buf + wf), s);
+    cudaFreeAsync(buf, s);
     return e;
 }
 
@@ -592,8 +775,8 @@ cudaError_t launch_norm2_acc(const float *v, int64_t n, double *out, cudaStream_
 // a process that reserved the GPU's memory up front for its own pool (a
 // cudaMalloc would fail or escape its accounting), or a latency-critical loop
 // where the device-wide synchronization of cudaFree is not acceptable. For
-// them the update's scratch (the float32 inverse of V, the column sums of
-// squares and their reciprocals) lives in one file-scope device array that
+// them the update's scratch (the float32 inverse of V and the column sums of
+// squares) lives in one file-scope device array that
 // every GPU which loads the library holds until the process exits.
 // ---------------------------------------------------------------------------
 namespace {
@@ -601,8 +784,7 @@ namespace {
 constexpr int kNoAllocMaxRank = 64;
 constexpr size_t kNoAllocWfBytes = sizeof(float) * kNoAllocMaxRank * kNoAllocMaxRank;
 constexpr size_t kNoAllocColsqOff = (kNoAllocWfBytes + 255) & ~size_t(255);
-constexpr size_t kNoAllocInvOff = kNoAllocColsqOff + ((sizeof(double) * kNoAllocMaxRank + 255) & ~size_t(255));
-constexpr size_t kNoAllocScratchBytes = kNoAllocInvOff + sizeof(float) * kNoAllocMaxRank;
+constexpr size_t kNoAllocScratchBytes = kNoAllocColsqOff + sizeof(double) * kNoAllocMaxRank;
 
 // Shared by every call on a device; holds the previous call's contents.
 static __device__ __align__(256) unsigned char g_update_scratch[kNoAllocScratchBytes];
@@ -679,33 +861,8 @@ cudaError_t launch_cpals_update_noalloc(const double *const *grams, int N, int m
     unsigned char *base = nullptr;
     cudaError_t e = update_scratch(&base);
     if (e != cudaSuccess) return e;
-    float *Wf = reinterpret_cast<float *>(base);
-    double *colsq = reinterpret_cast<double *>(base + kNoAllocColsqOff);
-    float *inv = reinterpret_cast<float *>(base + kNoAllocInvOff);
-    GramPtrs gp;
-    for (int k = 0; k < MAXN; ++k) gp.g[k] = k < N ? grams[k] : nullptr;
-    const size_t shm_solve = sizeof(double) * 2 * R * R;
-    e = cudaFuncSetAttribute(k_solve_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_solve);
-    if (e != cudaSuccess) return e;
-    k_solve_small<<<1, 256, shm_solve, s>>>(gp, N, mode, R, Wf, info);
-    e = cudaGetLastError();
-    if (e == cudaSuccess && I > 0) {
-        const size_t shm = sizeof(float) * (R * R + 8 * R);
-        e = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-        if (e == cudaSuccess) {
-            k_apply<<<grid_cap(I, 8), 256, shm, s>>>(M, I, R, Wf, A);
-            e = cudaGetLastError();
-        }
-    }
-    if (e == cudaSuccess) {
-        k_zero_d<<<1, 256, 0, s>>>(colsq, R);  // the shared scratch keeps the last call's sums
-        if (I > 0) k_colsq<<<grid_cap(I, 256 / R), 256, 0, s>>>(A, I, R, colsq);
-        k_sqrt_lambda<<<1, 128, 0, s>>>(colsq, R, lambda, inv);
-        if (I > 0) k_scale_cols<<<grid_cap(I * R, 256), 256, 0, s>>>(A, I, R, inv);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess && G_out) e = launch_gram(A, BLCO_F32, I, R, G_out, s);
-    return e;
+    return run_update(grams, N, mode, R, M, I, A, lambda, G_out, info, reinterpret_cast<float *>(base),
+                      reinterpret_cast<double *>(base + kNoAllocColsqOff), s);
 }
 
 }  // namespace blco
