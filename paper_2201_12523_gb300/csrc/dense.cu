@@ -64,7 +64,9 @@ __device__ __forceinline__ float to_f<__half>(__half v) { return __half2float(v)
 // Bound by the ten float32 operations per product. CTAs are as wide as whole
 // thread groups need (at most kGramThreads): with 256 threads, R = 64 left one
 // group of 136 threads and the other 120 idle, and 2^20 rows took 1.30 ms; two
-// groups in 288 threads take 1.09.
+// groups in 288 threads take 1.09 (packed f32x2 arithmetic: 1.18, that pipe's
+// rate; two CTAs per SM without the register limit: 1.02, but 7-10 % slower at
+// R = 16 and 50).
 constexpr int kGramRows = 32;  // rows staged in shared memory per step
 constexpr int kGramThreads = 288;
 
@@ -238,8 +240,19 @@ struct GramPtrs {
 // column through shared memory. Bound by the one SM's FP64 pipe at R = 64
 // (R^2 / 2 multiply-adds per step) and by the step's chain (reciprocal, two
 // barriers) at R = 32: Cholesky with one thread per column of the inverse took
-// 376 us at R = 64 and 129 us at R = 32, this 154 and 62.
+// 376 us at R = 64 and 129 us at R = 32, this 122 and 41 (with a float64 division
+// and a third barrier per step 154 and 62).
 // -------------------------------------------------------------------------
+// 1 / x to float64 rounding: Newton's iteration from the float reciprocal, whose
+// error (about 2^-23) squares twice; a float64 division is a longer chain.
+// Outside the floats' range, and where x is not positive, it is the division.
+__device__ __forceinline__ double reciprocal(double x) {
+    if (!(x > 1e-30 && x < 1e30)) return 1.0 / x;
+    double r = (double)(1.f / (float)x);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
 constexpr int kSolveThreads = 256;
 constexpr int kSolveMaxRank = 64;
 constexpr int kSolveSlots = (kSolveMaxRank * (kSolveMaxRank + 1) / 2 + kSolveThreads - 1) / kSolveThreads;
@@ -258,59 +271,69 @@ __global__ void __launch_bounds__(kSolveThreads) k_solve_small(const GramPtrs gp
             if (k != mode) v *= gp.g[k][p];
         V[p] = v;
     }
-    __shared__ double pd_tol, rcp;
-    __shared__ double col[kSolveMaxRank], colr[kSolveMaxRank];
+    __shared__ double pd_tol, rcp[2];
+    __shared__ double col[2][kSolveMaxRank], colr[kSolveMaxRank];
     __shared__ int ok;
     __syncthreads();
-    if (tid == 0) {
-        ok = 1;
+    if (tid < 32) {
         // smallest pivot accepted as positive: R * eps * max_i V_ii; at or
         // below it V is treated as not positive definite (numerically
         // singular or indefinite) and the pseudo-inverse is used
         double m = 0.0;
-        for (int i = 0; i < R; ++i) m = fmax(m, V[i * R + i]);
-        pd_tol = (double)R * 2.220446049250313e-16 * m;
+        for (int i = tid; i < R; i += 32) m = fmax(m, V[i * R + i]);
+        for (int o = 16; o >= 1; o >>= 1) m = fmax(m, __shfl_xor_sync(kFull, m, o));
+        if (tid == 0) {
+            ok = 1;
+            pd_tol = (double)R * 2.220446049250313e-16 * m;
+        }
     }
     // entry (row, column) of the lower triangle in slot q of this thread
     const int ntri = R * (R + 1) / 2;
+    const int slots = (ntri + kSolveThreads - 1) / kSolveThreads;
     double x[kSolveSlots];
     int ri[kSolveSlots], ci[kSolveSlots];
 #pragma unroll
     for (int q = 0; q < kSolveSlots; ++q) {
         const int t = tid + q * kSolveThreads;
-        int i = 0, rest = t;
-        while (rest > i) {
-            rest -= i + 1;
-            ++i;
-        }
+        int i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);  // row, up to rounding
+        if (i * (i + 1) / 2 > t) --i;
+        if ((i + 1) * (i + 2) / 2 <= t) ++i;
         ri[q] = t < ntri ? i : -1;
-        ci[q] = t < ntri ? rest : -1;
-        x[q] = t < ntri ? V[i * R + rest] : 0.0;
+        ci[q] = t < ntri ? t - i * (i + 1) / 2 : -1;
+        x[q] = t < ntri ? V[ri[q] * R + ci[q]] : 0.0;
     }
-    for (int j = 0; j < R; ++j) {
-        // the pivot's row and column
-#pragma unroll
-        for (int q = 0; q < kSolveSlots; ++q) {
-            if (ci[q] == j) col[ri[q]] = x[q];
-            else if (ri[q] == j) col[ci[q]] = x[q];
-            if (ri[q] == j && ci[q] == j) rcp = 1.0 / x[q];
+    // passes on the part of row and column j that slot q holds
+    const auto publish = [&](int q, int j) {
+        if (ci[q] == j) {
+            col[j & 1][ri[q]] = x[q];
+            if (ri[q] == j) rcp[j & 1] = reciprocal(x[q]);
+        } else if (ri[q] == j) {
+            col[j & 1][ci[q]] = x[q];
         }
-        __syncthreads();
+    };
+#pragma unroll
+    for (int q = 0; q < kSolveSlots; ++q)
+        if (q < slots) publish(q, 0);
+    __syncthreads();
+    for (int j = 0; j < R; ++j) {
+        const double *c = col[j & 1];
+        const double d = rcp[j & 1];
         if (tid < R) {
-            colr[tid] = col[tid] * rcp;
-            if (tid == j && !(col[j] > pd_tol)) ok = 0;
+            colr[tid] = c[tid] * d;
+            if (tid == j && !(c[j] > pd_tol)) ok = 0;
         }
         __syncthreads();
         if (!ok) break;
 #pragma unroll
         for (int q = 0; q < kSolveSlots; ++q) {
-            if (ri[q] < 0) continue;
+            if (q >= slots || ri[q] < 0) continue;
             if (ri[q] == j)
-                x[q] = ci[q] == j ? -rcp : colr[ci[q]];
+                x[q] = ci[q] == j ? -d : colr[ci[q]];
             else if (ci[q] == j)
                 x[q] = colr[ri[q]];
             else
-                x[q] = fma(-colr[ri[q]], col[ci[q]], x[q]);
+                x[q] = fma(-colr[ri[q]], c[ci[q]], x[q]);
+            publish(q, j + 1);
         }
         __syncthreads();
     }
