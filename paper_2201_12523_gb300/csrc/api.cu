@@ -213,9 +213,8 @@ void release(blco_tensor *h) {
     h->dfree(h->d_vals64, 0);
     h->dfree(h->d_perm, 0);
     h->dfree(h->d_bstart, 0);
-    h->dfree(h->d_bbase, 0);
     h->dfree(h->d_tile_block, 0);
-    for (int n = 0; n < MAXN; ++n) h->dfree(h->d_hot[n], 0);
+    h->dfree(h->d_hot[0], 0);  // one allocation for all modes
     h->dfree(h->d_order, 0);
     for (int q = 0; q < 8; ++q) {
         h->dfree(h->q_keys[q], 0);
@@ -481,7 +480,8 @@ bool copy_buffer(blco_tensor *h, size_t bytes, float **p) {
 }
 
 blco_status mttkrp_device(blco_tensor *h, int mode, const FactorSet &fs, blco_dtype fdt, int R, float *out,
-                          const float *vals_ext, cudaStream_t s, int64_t range_begin = 0, int64_t range_end = -1) {
+                          const float *vals_ext, cudaStream_t s, int64_t range_begin = 0, int64_t range_end = -1,
+                          bool zeroed = false) {
     const int64_t n = h->L.dims[mode] * (int64_t)R;
     const HotRows hot = hot_for(h, mode, R);
     // short modes: reduce into one private copy per SM, then sum the copies
@@ -494,7 +494,8 @@ blco_status mttkrp_device(blco_tensor *h, int mode, const FactorSet &fs, blco_dt
     } else {
         dst = out;
     }
-    cudaError_t e = timed(h, "zero", s, [&]() { return launch_zero(dst, n * oc.n, s); });
+    cudaError_t e = cudaSuccess;
+    if (!zeroed || dst != out) e = timed(h, "zero", s, [&]() { return launch_zero(dst, n * oc.n, s); });
     if (e != cudaSuccess) return cuda_fail(e, "zero output");
     const bool tiled = h->d_order && range_end < 0 && !(h->compensated && fdt != BLCO_F32);
     blco_status st = over_store(
@@ -634,8 +635,9 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
         for (int64_t b = 0; b < nb; ++b)
             for (int n = 0; n < N; ++n)
                 bbase[b * MAXN + n] = h->L.width[n] >= 32 ? 0u : (h->bhigh[b * N + n] << h->L.width[n]);
-        e = h->dalloc((void **)&h->d_bstart, sizeof(int64_t) * (nb + 1));
-        if (e == cudaSuccess) e = h->dalloc((void **)&h->d_bbase, sizeof(uint32_t) * bbase.size());
+        // one allocation: block offsets, then high bits
+        e = h->dalloc((void **)&h->d_bstart, sizeof(int64_t) * (nb + 1) + sizeof(uint32_t) * bbase.size());
+        if (e == cudaSuccess) h->d_bbase = reinterpret_cast<uint32_t *>(h->d_bstart + nb + 1);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(h->d_bstart, h->bstart.data(), sizeof(int64_t) * (nb + 1), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess)
@@ -649,16 +651,20 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
     // hot rows per mode (histogram of the stored indices, top counts)
     if (nnz > 0) {
         uint32_t *counts = nullptr;
+        // as many rows as the smallest supported rank can hold on chip
+        size_t rows = 0;
+        for (int n = 0; n < N; ++n) {
+            h->hot_count[n] = (int)std::min<int64_t>(h->L.dims[n], warp_tier_capacity(8));
+            rows += h->hot_count[n];
+        }
+        e = h->dalloc((void **)&h->d_hot[0], sizeof(uint32_t) * rows);
         for (int n = 0; n < N && e == cudaSuccess; ++n) {
             const int64_t I = h->L.dims[n];
-            // as many rows as the smallest supported rank can hold on chip
-            const int k = (int)std::min<int64_t>(I, warp_tier_capacity(8));
+            if (n > 0) h->d_hot[n] = h->d_hot[n - 1] + h->hot_count[n - 1];
             e = cudaMallocAsync(&counts, sizeof(uint32_t) * I, s);
             if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, sizeof(uint32_t) * I, s);
             if (e == cudaSuccess) e = mode_histogram(h->view(), n, counts, s);
-            if (e == cudaSuccess) e = h->dalloc((void **)&h->d_hot[n], sizeof(uint32_t) * k);
-            if (e == cudaSuccess) e = top_rows(counts, I, k, h->d_hot[n], s);
-            h->hot_count[n] = k;
+            if (e == cudaSuccess) e = top_rows(counts, I, h->hot_count[n], nnz, h->d_hot[n], s);
             if (counts) cudaFreeAsync(counts, s);
             counts = nullptr;
         }
@@ -743,7 +749,7 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
     if (!h->streamed && h->budget == 0 && tile_order_supported(h->L) && nnz >= kOrderMinNnz) {
         const size_t ob = tile_order_bytes(nnz, N, no_vals);
         size_t free_b = 0, total_b = 0;
-        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && ob <= free_b / 4 &&
+        if ((ob <= ((size_t)16 << 20) || (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && ob <= free_b / 4)) &&
             h->dalloc(&h->d_order, ob) == cudaSuccess) {
             h->order = tile_order_view(h->d_order, nnz, N, no_vals);
             HotRows hot[MAXN];
@@ -1120,9 +1126,26 @@ blco_status blco_mttkrp_all(blco_handle h, const void *const *factors, blco_dtyp
     if (fused || (h->streamed && !h->host_reads))
         return mttkrp_all_onepass(h, fs, host_in, host_out, in_off, out_off, total, fdt, R, outs, s, fused);
     if (total == 0) {  // device arguments: the modes one after another on s
+        // every output zeroed by one launch, unless one of them shares memory
+        // with a factor that an earlier mode still gathers
+        int64_t len[MAXN] = {};
+        bool apart = true;
         for (int n = 0; n < N; ++n) {
             if (!outs[n]) continue;
-            st = mttkrp_device(h, n, fs, fdt, R, outs[n], nullptr, s);
+            len[n] = h->L.dims[n] * (int64_t)R;
+            const uintptr_t o0 = reinterpret_cast<uintptr_t>(outs[n]), o1 = o0 + len[n] * sizeof(float);
+            for (int k = 0; k < N; ++k) {
+                const uintptr_t f0 = reinterpret_cast<uintptr_t>(factors[k]);
+                apart &= o1 <= f0 || f0 + h->L.dims[k] * (int64_t)R * dtype_size(fdt) <= o0;
+            }
+        }
+        if (apart) {
+            cudaError_t e = timed(h, "zero", s, [&]() { return launch_zero_list(outs, len, N, s); });
+            if (e != cudaSuccess) return cuda_fail(e, "zero outputs");
+        }
+        for (int n = 0; n < N; ++n) {
+            if (!outs[n]) continue;
+            st = mttkrp_device(h, n, fs, fdt, R, outs[n], nullptr, s, 0, -1, apart);
             if (st != BLCO_OK) return st;
         }
         return BLCO_OK;

@@ -659,6 +659,35 @@ cudaError_t launch_zero(float *p, int64_t n, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+namespace {
+struct ZeroList {
+    float4 *p[MAXN];
+    int64_t n4[MAXN];
+};
+__global__ void k_zero_list(const ZeroList z) {
+    float4 *p = z.p[blockIdx.y];
+    const int64_t n4 = z.n4[blockIdx.y];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x)
+        p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+}  // namespace
+
+// Zeroes several 16-byte aligned arrays, of multiples of 4 floats, in one launch.
+cudaError_t launch_zero_list(float *const *p, const int64_t *n, int count, cudaStream_t s) {
+    ZeroList z = {};
+    int64_t longest = 0;
+    int used = 0;
+    for (int i = 0; i < count; ++i) {
+        if (!p[i] || n[i] <= 0) continue;
+        z.p[used] = reinterpret_cast<float4 *>(p[i]);
+        z.n4[used++] = n[i] / 4;
+        longest = std::max(longest, n[i] / 4);
+    }
+    if (used == 0) return cudaSuccess;
+    k_zero_list<<<dim3(grid_cap(longest, 256), (unsigned)used), 256, 0, s>>>(z);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_convert(const float *src, void *dst, blco_dtype dt, int64_t n, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     if (dt == BLCO_BF16)

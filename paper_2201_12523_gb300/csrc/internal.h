@@ -154,11 +154,13 @@ cudaError_t build_tile_block(const int64_t *d_bstart, int64_t nblocks, int64_t n
                              uint32_t *tile_block, cudaStream_t s);
 // Per-mode index histogram of the store's nonzeros (counts: I_n uint32).
 cudaError_t mode_histogram(const StoreView &sv, int mode, uint32_t *counts, cudaStream_t s);
-// The `k` rows with the largest counts (ties: lower row id), sorted by row id.
-cudaError_t top_rows(const uint32_t *counts, int64_t I, int k, uint32_t *rows_out, cudaStream_t s);
+// The `k` rows with the largest counts (ties: lower row id), by decreasing
+// count; no count exceeds `most`.
+cudaError_t top_rows(const uint32_t *counts, int64_t I, int k, int64_t most, uint32_t *rows_out, cudaStream_t s);
 
 // dense.cu
 cudaError_t launch_zero(float *p, int64_t n, cudaStream_t s);
+cudaError_t launch_zero_list(float *const *p, const int64_t *n, int count, cudaStream_t s);
 cudaError_t launch_sum_copies(const float *copies, int ncopies, int64_t n, float *out, cudaStream_t s);
 cudaError_t launch_convert(const float *src, void *dst, blco_dtype dt, int64_t n, cudaStream_t s);
 cudaError_t launch_gram(const void *A, blco_dtype fdt, int64_t I, int R, double *G, cudaStream_t s);

@@ -35,6 +35,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "mttkrp_kernels.cuh"
 
@@ -573,10 +574,32 @@ TParams tiled_params(const StoreView &sv, const TileOrder &to, const void *const
     return p;
 }
 
+// Clusters of a kernel that are resident at once with `shm` bytes of shared
+// memory (a cluster stays inside a GPC, so that is not the SMs' CTAs over the
+// cluster's size). The query costs as much as a launch: each kernel remembers
+// its last answer, with the device and the size it was for.
 template <typename K>
-cudaError_t launch_tiled(K kern, const TParams &p, size_t shm, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-    if (e != cudaSuccess) return e;
+int resident_clusters(K kern, const cudaLaunchConfig_t &cfg, std::atomic<uint64_t> &last) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
+    const uint64_t tag = ((uint64_t)(dev & 0xFF) << 24 | (cfg.dynamicSmemBytes & 0xFFFFFF)) << 32;
+    const uint64_t seen = last.load(std::memory_order_relaxed);
+    if ((seen & ~0xFFFFFFFFull) == tag && (uint32_t)seen != 0) return (int)(uint32_t)seen;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
+        cudaGetLastError();
+        return 1;
+    }
+    last.store(tag | (uint32_t)clusters, std::memory_order_relaxed);
+    return clusters;
+}
+
+template <typename K>
+cudaError_t launch_tiled(K kern, const TParams &p, size_t shm, std::atomic<uint64_t> &last, cudaStream_t s) {
+    if (shm > 48 * 1024) {  // what a kernel may use without asking
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+        if (e != cudaSuccess) return e;
+    }
     const int64_t tiles = (p.nnz + kTile - 1) / kTile;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kTiledCluster);
@@ -589,24 +612,19 @@ cudaError_t launch_tiled(K kern, const TParams &p, size_t shm, cudaStream_t s) {
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    // as many clusters as are resident at once (a cluster stays inside a GPC, so
-    // that is not the SMs' CTAs over the cluster's size), or as have a tile
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
-        cudaGetLastError();
-        clusters = 1;
-    }
     const int64_t need = (tiles + kTiledCluster - 1) / kTiledCluster;
-    cfg.gridDim = dim3((unsigned)(std::min<int64_t>(clusters, need) * kTiledCluster));
+    cfg.gridDim = dim3((unsigned)(std::min<int64_t>(resident_clusters(kern, cfg, last), need) * kTiledCluster));
     return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
 template <typename T, int R, int NG>
 cudaError_t run_tiled(const TParams &p, cudaStream_t s) {
     constexpr int P = kTile / (kTiledThreads / (R / lane_vec<T, R>()));
+    static std::atomic<uint64_t> last{0};
     return launch_tiled(
         k_mttkrp_tiled<T, R, NG>, p,
-        tiled_smem(sizeof(uint4), staged<P>(), p.n_inner > 1 ? p.n_inner - 1 : 0, p.kw, R * sizeof(float)).total, s);
+        tiled_smem(sizeof(uint4), staged<P>(), p.n_inner > 1 ? p.n_inner - 1 : 0, p.kw, R * sizeof(float)).total, last,
+        s);
 }
 
 template <typename T, int R>
@@ -640,10 +658,11 @@ cudaError_t tiled_as(const StoreView &sv, const TileOrder &to, const FactorSet &
 template <int R, int NG>
 cudaError_t run_tiled64(const TParams &p, cudaStream_t s) {
     constexpr int P = kTile / (kTiledThreads / (R < 32 ? R : 32));
+    static std::atomic<uint64_t> last{0};
     return launch_tiled(
         k_mttkrp64_tiled<R, NG>, p,
         tiled_smem(sizeof(Rec64), staged<P>(), (p.n_inner > 1 ? p.n_inner - 1 : 0) + 1, p.kw, R * sizeof(double)).total,
-        s);
+        last, s);
 }
 
 template <int R>
