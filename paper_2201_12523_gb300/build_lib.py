@@ -47,7 +47,7 @@ def _stale(target: str, deps) -> bool:
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
     headers = [os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "mttkrp_kernels.cuh"),
-               os.path.join(CSRC, "mttkrp_tiled.cuh"), os.path.join(CSRC, "hot_rows.cuh"),
+               os.path.join(CSRC, "mttkrp_tiled.cuh"), os.path.join(CSRC, "hot_rows.cuh"), os.path.join(CSRC, "tile_stage.cuh"),
                os.path.join(INCLUDE, "blco.h")]
     objs, jobs = [], []
     for src in SOURCES:

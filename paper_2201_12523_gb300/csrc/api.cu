@@ -1063,7 +1063,10 @@ static blco_status mttkrp_all_onepass(blco_tensor *h, FactorSet fs, const bool *
     blco_status st = over_store(h, nullptr, nullptr, s, [&](const StoreView &sv, cudaStream_t q) {
         if (fused)
             return timed(h, "mttkrp_all_fused", q,
-                         [&]() { return launch_mttkrp_fused(sv, fs, fdt, R, hot_all, dst_all, q); });
+                         [&]() {
+                             return launch_mttkrp_fused(sv, h->d_order ? &h->order : nullptr, fs, fdt, R, hot_all,
+                                                        dst_all, q);
+                         });
         for (int n = 0; n < N; ++n) {
             if (!outs[n]) continue;
             cudaError_t e = timed(h, "mttkrp", q, [&]() {

@@ -108,8 +108,9 @@ bool rank_supported(int R);
 // store's shape and the rank allow it (5 modes, every I_n <= 2^24,
 // R = 16, 32 or 64).
 bool fused_supported(const StoreView &sv, int R);
-cudaError_t launch_mttkrp_fused(const StoreView &sv, const FactorSet &fs, blco_dtype fdt, int R, const HotRows *hot,
-                                float *const *outs, cudaStream_t s);
+// `to`: the store's order inside tiles, or NULL.
+cudaError_t launch_mttkrp_fused(const StoreView &sv, const TileOrder *to, const FactorSet &fs, blco_dtype fdt, int R,
+                                const HotRows *hot, float *const *outs, cudaStream_t s);
 // tile_order.cu
 int order_partner(const int64_t *dims, int N, int mode);
 bool tile_order_supported(const Layout &L);  // at least two modes, of at most 2^31 rows each

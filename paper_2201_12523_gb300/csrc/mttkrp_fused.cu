@@ -26,7 +26,10 @@
 // at 5 modes it runs 1.4-1.7x faster than five per-mode launches; at 3 and 4
 // modes the per-mode kernels (sorted tiles, 2 or 3 gathers per nonzero) are
 // as fast or faster, and blco_mttkrp_all uses them there.
+#include <algorithm>
+
 #include "mttkrp_kernels.cuh"
+#include "tile_stage.cuh"
 
 namespace blco {
 namespace {
@@ -60,6 +63,8 @@ struct FusedParams {
     int table_off[MAXN];          // bucket offset of mode n's table
     int warp_floats;              // floats of one warp's copies (all modes)
     int table_buckets;            // buckets of all tables
+    const uint16_t *rank[MAXN];   // order inside tiles: rank | place among the hottest rows << 10
+    int order_mode;               // the mode whose ranks order the tiles
 };
 
 template <int N>
@@ -68,9 +73,17 @@ struct FStage {
     float val[32];
 };
 
-__host__ __device__ __forceinline__ size_t fused_smem(int N, int warp_floats, int buckets) {
-    const size_t stage = align16((size_t)(N + 1) * 32 * sizeof(uint32_t)) * kWarps;
-    return align16(stage + (size_t)kWarps * warp_floats * sizeof(float)) + (size_t)buckets * sizeof(uint4);
+// Shared memory: staging, copies, a claim word per copied row, tables.
+struct FusedSmem {
+    size_t wacc, claim, table, total;
+};
+__host__ __device__ __forceinline__ FusedSmem fused_smem(int N, int R, int warp_floats, int buckets) {
+    FusedSmem L;
+    L.wacc = align16((size_t)(N + 1) * 32 * sizeof(uint32_t)) * kWarps;
+    L.claim = L.wacc + (size_t)kWarps * warp_floats * sizeof(float);
+    L.table = align16(L.claim + (size_t)kWarps * (warp_floats / R) * sizeof(uint32_t));
+    L.total = L.table + (size_t)buckets * sizeof(uint4);
+    return L;
 }
 
 template <int R, int VEC, int H>
@@ -101,6 +114,157 @@ __device__ __forceinline__ uint32_t fused_block_of(const uint32_t *tile_block, c
     return b;
 }
 
+// One subgroup's walk over STEPS staged positions, `live` of them nonzeros (the
+// others end the staged range): per mode a running sum while the row stays the
+// same, stored where it changes and at the end. `id` is mode 0's first staged
+// word, the modes `stride` apart. Called by whole warps.
+template <typename T, int R, int N, int STEPS, int UNROLL>
+__device__ __forceinline__ void walk_range(const FusedParams &p, const char *const (&rowp)[N], const uint32_t *id,
+                                           int stride, const float *val, int live, float *wacc, uint32_t *claim, int g,
+                                           int c) {
+    constexpr int VEC = lane_vec<T, R>();
+    constexpr int H = VEC / 2;
+    constexpr int CH = 1;  // positions whose rows load back to back
+    uint32_t cur[N];
+    f2 acc[N][H];
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        cur[n] = kRunNone;
+#pragma unroll
+        for (int h = 0; h < H; ++h) acc[n][h] = 0ull;
+    }
+    // stores the open run of every mode with flush[n] set: cold rows by
+    // vector reductions, hot rows by read-modify-write of the warp's copy,
+    // one subgroup at a time (warp-uniform call)
+    auto store_runs = [&](const bool (&flush)[N]) {
+        unsigned pending = 0;  // modes with a hot run to store
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            if (!flush[n] || !p.out[n]) continue;
+            if ((cur[n] >> 24) == kSlotNone)
+                fused_red_global<R, VEC, H>(p.out[n], cur[n] & kIdMask, c, acc[n]);
+            else
+                pending |= 1u << n;
+        }
+        // every subgroup claims its rows, the last claim of a row stands;
+        // whose claim stands updates the copy, the others claim again
+        while (__any_sync(kFull, pending != 0)) {
+#pragma unroll
+            for (int n = 0; n < N; ++n)
+                if (pending & (1u << n)) claim[p.wacc_off[n] / R + (cur[n] >> 24)] = (uint32_t)g;
+            __syncwarp();
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+                if (!(pending & (1u << n))) continue;
+                const int row = p.wacc_off[n] / R + (int)(cur[n] >> 24);
+                if (claim[row] != (uint32_t)g) continue;
+                fused_rmw<VEC, H>(wacc + (size_t)row * R + c * VEC, acc[n]);
+                pending &= ~(1u << n);
+            }
+            __syncwarp();
+        }
+    };
+#pragma unroll UNROLL
+    for (int j0 = 0; j0 < STEPS; j0 += CH) {
+        uint32_t w[CH][N];
+        f2 pre[CH][H];  // value times the rows of modes before n
+#pragma unroll
+        for (int i = 0; i < CH; ++i) {
+            const float v = val[j0 + i];
+#pragma unroll
+            for (int n = 0; n < N; ++n) w[i][n] = id[n * stride + j0 + i];
+            const f2 vv = pack2(v, v);
+#pragma unroll
+            for (int h = 0; h < H; ++h) pre[i][h] = vv;
+        }
+        f2 rowv[CH][N][H];
+#pragma unroll
+        for (int n = 0; n < N; ++n)
+#pragma unroll
+            for (int i = 0; i < CH; ++i)
+                Chunk<T>::load(rowp[n] + (size_t)(w[i][n] & kIdMask) * (R * sizeof(T)), rowv[i][n]);
+#pragma unroll
+        for (int i = 0; i < CH; ++i) {
+            const bool in = j0 + i < live;
+            // products for every mode: prefix (value and modes < n) times suffix (modes > n)
+            f2 prod[N][H];
+            {
+                f2 run[H];
+#pragma unroll
+                for (int h = 0; h < H; ++h) run[h] = pre[i][h];
+#pragma unroll
+                for (int n = 0; n < N; ++n) {
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        prod[n][h] = run[h];
+                        run[h] = mul2(run[h], rowv[i][n][h]);
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < H; ++h) run[h] = rowv[i][N - 1][h];
+#pragma unroll
+                for (int n = N - 2; n >= 0; --n) {
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        prod[n][h] = mul2(prod[n][h], run[h]);
+                        if (n > 0) run[h] = mul2(run[h], rowv[i][n][h]);
+                    }
+                }
+            }
+            bool flush[N];
+#pragma unroll
+            for (int n = 0; n < N; ++n) flush[n] = in && cur[n] != kRunNone && w[i][n] != cur[n];
+            store_runs(flush);
+            if (in) {
+#pragma unroll
+                for (int n = 0; n < N; ++n) {
+                    if (cur[n] == kRunNone || w[i][n] != cur[n]) {
+                        cur[n] = w[i][n];
+#pragma unroll
+                        for (int h = 0; h < H; ++h) acc[n][h] = prod[n][h];
+                    } else {
+#pragma unroll
+                        for (int h = 0; h < H; ++h) acc[n][h] = add2(acc[n][h], prod[n][h]);
+                    }
+                }
+            }
+        }
+    }
+    // the range's open runs
+    {
+        bool flush[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) flush[n] = cur[n] != kRunNone;
+        store_runs(flush);
+    }
+}
+
+// Adds the CTA's per-warp copies to the outputs once.
+template <int R, int N>
+__device__ __forceinline__ void merge_copies(const FusedParams &p, const float *wacc_all) {
+    constexpr int Q = R / 4;
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        if (!p.out[n]) continue;
+        for (int i = threadIdx.x; i < p.kw[n] * Q; i += kThreads) {
+            const int sl = i / Q, q = i % Q;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int ww = 0; ww < kWarps; ++ww) {
+                const float4 x = *reinterpret_cast<const float4 *>(wacc_all + (size_t)ww * p.warp_floats + p.wacc_off[n] +
+                                                                   (size_t)sl * R + q * 4);
+                v.x += x.x;
+                v.y += x.y;
+                v.z += x.z;
+                v.w += x.w;
+            }
+            const uint32_t row = p.hot_dense[n] ? (uint32_t)sl : __ldg(p.hot_rows[n] + sl);
+            if (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f)
+                red_add_v4(p.out[n] + (size_t)row * R + q * 4, v.x, v.y, v.z, v.w);
+        }
+    }
+}
+
 template <typename T, int R, int N>
 __host__ __device__ constexpr int fused_min_ctas() {
     return 2;
@@ -114,7 +278,6 @@ __global__ void __launch_bounds__(kThreads, fused_min_ctas<T, R, N>()) k_mttkrp_
     static_assert(G >= 1 && G <= 32 && (32 % G) == 0, "rank must give 1..32 lanes per row");
     static_assert(H % 2 == 0, "the shared-copy update moves 16 bytes at a time");
     constexpr int STEPS = G;
-    constexpr int CH = 1;  // positions whose rows load back to back
 
     extern __shared__ __align__(16) unsigned char smem[];
     const size_t stage_bytes = align16((size_t)(N + 1) * 32 * sizeof(uint32_t));
@@ -123,10 +286,11 @@ __global__ void __launch_bounds__(kThreads, fused_min_ctas<T, R, N>()) k_mttkrp_
     const int g = lane / G;
     const int c = lane % G;
     FStage<N> &st = *reinterpret_cast<FStage<N> *>(smem + stage_bytes * wid);
-    float *wacc_all = reinterpret_cast<float *>(smem + stage_bytes * kWarps);
+    const FusedSmem L = fused_smem(N, R, p.warp_floats, p.table_buckets);
+    float *wacc_all = reinterpret_cast<float *>(smem + L.wacc);
     float *wacc = wacc_all + (size_t)wid * p.warp_floats;
-    uint4 *tables =
-        reinterpret_cast<uint4 *>(smem + align16(stage_bytes * kWarps + (size_t)kWarps * p.warp_floats * sizeof(float)));
+    uint32_t *claim = reinterpret_cast<uint32_t *>(smem + L.claim) + wid * (p.warp_floats / R);
+    uint4 *tables = reinterpret_cast<uint4 *>(smem + L.table);
 
     // --- zero the copies; thread n fills mode n's table in order of decreasing count
     for (int i = threadIdx.x; i < kWarps * p.warp_floats; i += kThreads) wacc_all[i] = 0.f;
@@ -205,119 +369,8 @@ __global__ void __launch_bounds__(kThreads, fused_min_ctas<T, R, N>()) k_mttkrp_
         __syncwarp();
 
         // --- subgroup g walks positions [g*G, g*G+G) in store order
-        uint32_t cur[N];
-        f2 acc[N][H];
-#pragma unroll
-        for (int n = 0; n < N; ++n) {
-            cur[n] = kRunNone;
-#pragma unroll
-            for (int h = 0; h < H; ++h) acc[n][h] = 0ull;
-        }
-        // stores the open run of every mode with flush[n] set: cold rows by
-        // vector reductions, hot rows by read-modify-write of the warp's copy,
-        // one subgroup at a time (warp-uniform call)
-        auto store_runs = [&](const bool (&flush)[N]) {
-            bool hot_pending = false;
-#pragma unroll
-            for (int n = 0; n < N; ++n) {
-                if (!flush[n] || !p.out[n]) continue;
-                const uint32_t sl = cur[n] >> 24;
-                if (sl == kSlotNone) {
-                    fused_red_global<R, VEC, H>(p.out[n], cur[n] & kIdMask, c, acc[n]);
-                } else {
-                    hot_pending = true;
-                }
-            }
-            unsigned pend = __ballot_sync(kFull, hot_pending);
-            while (pend) {
-                const int sg = (__ffs(pend) - 1) / G;
-                if (g == sg && hot_pending) {
-#pragma unroll
-                    for (int n = 0; n < N; ++n) {
-                        if (!flush[n] || !p.out[n]) continue;
-                        const uint32_t sl = cur[n] >> 24;
-                        if (sl != kSlotNone) fused_rmw<VEC, H>(wacc + p.wacc_off[n] + (size_t)sl * R + c * VEC, acc[n]);
-                    }
-                }
-                __syncwarp();
-                pend &= ~((G == 32 ? kFull : ((1u << G) - 1u)) << (sg * G));
-            }
-        };
-#pragma unroll
-        for (int j0 = 0; j0 < STEPS; j0 += CH) {
-            uint32_t w[CH][N];
-            f2 pre[CH][H];  // value times the rows of modes before n
-#pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                const int s = g * STEPS + j0 + i;
-                const float v = st.val[s];
-#pragma unroll
-                for (int n = 0; n < N; ++n) w[i][n] = st.id[n][s];
-                const f2 vv = pack2(v, v);
-#pragma unroll
-                for (int h = 0; h < H; ++h) pre[i][h] = vv;
-            }
-            f2 rowv[CH][N][H];
-#pragma unroll
-            for (int n = 0; n < N; ++n)
-#pragma unroll
-                for (int i = 0; i < CH; ++i)
-                    Chunk<T>::load(rowp[n] + (size_t)(w[i][n] & kIdMask) * (R * sizeof(T)), rowv[i][n]);
-#pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                const int s = g * STEPS + j0 + i;
-                const bool in = s < nvalid;
-                // products for every mode: prefix (value and modes < n) times suffix (modes > n)
-                f2 prod[N][H];
-                {
-                    f2 run[H];
-#pragma unroll
-                    for (int h = 0; h < H; ++h) run[h] = pre[i][h];
-#pragma unroll
-                    for (int n = 0; n < N; ++n) {
-#pragma unroll
-                        for (int h = 0; h < H; ++h) {
-                            prod[n][h] = run[h];
-                            run[h] = mul2(run[h], rowv[i][n][h]);
-                        }
-                    }
-#pragma unroll
-                    for (int h = 0; h < H; ++h) run[h] = rowv[i][N - 1][h];
-#pragma unroll
-                    for (int n = N - 2; n >= 0; --n) {
-#pragma unroll
-                        for (int h = 0; h < H; ++h) {
-                            prod[n][h] = mul2(prod[n][h], run[h]);
-                            if (n > 0) run[h] = mul2(run[h], rowv[i][n][h]);
-                        }
-                    }
-                }
-                bool flush[N];
-#pragma unroll
-                for (int n = 0; n < N; ++n) flush[n] = in && cur[n] != kRunNone && w[i][n] != cur[n];
-                store_runs(flush);
-                if (in) {
-#pragma unroll
-                    for (int n = 0; n < N; ++n) {
-                        if (cur[n] == kRunNone || w[i][n] != cur[n]) {
-                            cur[n] = w[i][n];
-#pragma unroll
-                            for (int h = 0; h < H; ++h) acc[n][h] = prod[n][h];
-                        } else {
-#pragma unroll
-                            for (int h = 0; h < H; ++h) acc[n][h] = add2(acc[n][h], prod[n][h]);
-                        }
-                    }
-                }
-            }
-        }
-        // the range's open runs
-        {
-            bool flush[N];
-#pragma unroll
-            for (int n = 0; n < N; ++n) flush[n] = cur[n] != kRunNone;
-            store_runs(flush);
-        }
+        walk_range<T, R, N, STEPS, STEPS>(p, rowp, &st.id[0][g * STEPS], 32, &st.val[g * STEPS], nvalid - g * STEPS,
+                                          wacc, claim, g, c);
         __syncwarp();
         tile = ntile;
         key = nkey;
@@ -326,27 +379,74 @@ __global__ void __launch_bounds__(kThreads, fused_min_ctas<T, R, N>()) k_mttkrp_
 
     // --- add the CTA's per-warp copies to the outputs once
     __syncthreads();
-    constexpr int Q = R / 4;
+    merge_copies<R, N>(p, wacc_all);
+}
+
+// The same walk over the order inside tiles (tile_order.cu) of a resident store:
+// a CTA stages a tile of kTile positions at their ranks by the longest mode's
+// row, so that this mode's runs and, inside them, those of the others last
+// longer than in store order, and a subgroup walks R ranks instead of R / 4
+// positions. Slots come with the ranks: no tables. 100M nonzeros of the 5-mode
+// Zipf shape, R = 16: 8.95 -> @FT@ ms.
+template <typename T, int R, int N>
+__global__ void __launch_bounds__(kThreads, 2) k_mttkrp_fused_tiled(const FusedParams p) {
+    constexpr int VEC = lane_vec<T, R>();
+    constexpr int G = R / VEC;
+    constexpr int P = kTile / (kThreads / G);
+    constexpr int S = staged<P>();
+    constexpr int PER = kTile / kThreads;
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint32_t *ids = reinterpret_cast<uint32_t *>(smem);  // [N][S]
+    float *vals = reinterpret_cast<float *>(ids + N * S);
+    float *wacc_all = vals + S;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int g = lane / G, c = lane % G;
+    const int sub = threadIdx.x / G;
+    float *wacc = wacc_all + (size_t)wid * p.warp_floats;
+    uint32_t *claim = reinterpret_cast<uint32_t *>(wacc_all + kWarps * p.warp_floats) + wid * (p.warp_floats / R);
+    for (int i = threadIdx.x; i < kWarps * p.warp_floats; i += kThreads) wacc_all[i] = 0.f;
+    const char *rowp[N];
 #pragma unroll
-    for (int n = 0; n < N; ++n) {
-        if (!p.out[n]) continue;
-        for (int i = threadIdx.x; i < p.kw[n] * Q; i += kThreads) {
-            const int sl = i / Q, q = i % Q;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int n = 0; n < N; ++n) rowp[n] = static_cast<const char *>(p.fac[n]) + (size_t)c * VEC * sizeof(T);
+
+    const int64_t ntiles = (p.end + kTile - 1) / kTile;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t base = tile * kTile;
+        const int nvalid = p.end - base < kTile ? (int)(p.end - base) : kTile;
+        if (threadIdx.x == 0 && tile + gridDim.x < ntiles - 1) {  // the next tile's arrays, to L2
+            const int64_t q = base + (int64_t)gridDim.x * kTile;
+            const auto ask = [](const void *a, int bytes) {
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(bytes));
+            };
+            ask(p.keys + q, kTile * (int)sizeof(uint64_t));
+            ask(p.vals + q, kTile * (int)sizeof(float));
 #pragma unroll
-            for (int ww = 0; ww < kWarps; ++ww) {
-                const float4 x = *reinterpret_cast<const float4 *>(wacc_all + (size_t)ww * p.warp_floats + p.wacc_off[n] +
-                                                                   (size_t)sl * R + q * 4);
-                v.x += x.x;
-                v.y += x.y;
-                v.z += x.z;
-                v.w += x.w;
-            }
-            const uint32_t row = p.hot_dense[n] ? (uint32_t)sl : __ldg(p.hot_rows[n] + sl);
-            if (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f)
-                red_add_v4(p.out[n] + (size_t)row * R + q * 4, v.x, v.y, v.z, v.w);
+            for (int n = 0; n < N; ++n) ask(p.rank[n] + q, kTile * (int)sizeof(uint16_t));
         }
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int q = threadIdx.x + i * kThreads;
+            const bool valid = q < nvalid;
+            const int64_t pos = base + q;
+            const uint64_t key = valid ? ld_stream_u64(p.keys + pos) : 0ull;
+            const uint32_t r = staged_at<P>(__ldcs(p.rank[p.order_mode] + pos) & (kTile - 1));
+            const uint32_t *bb = nullptr;
+            if (!p.single_block && valid) bb = p.bbase + (size_t)fused_block_of(p.tile_block, p.bstart, pos) * MAXN;
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+                const uint32_t place = __ldcs(p.rank[n] + pos) / kTile;
+                uint32_t row = (uint32_t)((key >> p.shift[n]) & p.mask[n]);
+                if (bb) row += __ldg(bb + n);
+                ids[n * S + r] = row | (place < (uint32_t)p.kw[n] ? place : kSlotNone) << 24;
+            }
+            vals[r] = valid ? ld_stream_f32(p.vals + pos) : 0.f;
+        }
+        __syncthreads();
+        walk_range<T, R, N, P, 1>(p, rowp, ids + sub * (P + 1), S, vals + sub * (P + 1), nvalid - sub * P, wacc, claim,
+                                  g, c);
+        __syncthreads();
     }
+    merge_copies<R, N>(p, wacc_all);
 }
 
 // Rows per warp on chip: 4 KB of float32 copies per warp, split over the modes.
@@ -354,7 +454,7 @@ constexpr int kFusedWarpBytes = 4 * 1024;
 
 template <typename T, int R, int N>
 cudaError_t run_fused(const FusedParams &p, cudaStream_t s) {
-    const size_t shm = fused_smem(N, p.warp_floats, p.table_buckets);
+    const size_t shm = fused_smem(N, R, p.warp_floats, p.table_buckets).total;
     auto kern = k_mttkrp_fused<T, R, N>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
     if (e != cudaSuccess) return e;
@@ -363,14 +463,31 @@ cudaError_t run_fused(const FusedParams &p, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+template <typename T, int R, int N>
+cudaError_t run_fused_tiled(const FusedParams &p, cudaStream_t s) {
+    constexpr int P = kTile / (kThreads / (R / lane_vec<T, R>()));
+    const size_t shm = (size_t)(N + 1) * staged<P>() * sizeof(uint32_t) +
+                       (size_t)kWarps * (p.warp_floats * sizeof(float) + p.warp_floats / R * sizeof(uint32_t));
+    auto kern = k_mttkrp_fused_tiled<T, R, N>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, shm) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    const int64_t tiles = (p.end + kTile - 1) / kTile;
+    kern<<<(unsigned)std::min<int64_t>((int64_t)sm_count() * per_sm, tiles), kThreads, shm, s>>>(p);
+    return cudaGetLastError();
+}
+
 template <typename T, int R>
 cudaError_t fused_by_n(const FusedParams &p, int N, cudaStream_t s) {
-    return N == kFusedModes ? run_fused<T, R, kFusedModes>(p, s) : cudaErrorInvalidValue;
+    if (N != kFusedModes) return cudaErrorInvalidValue;
+    return p.rank[0] ? run_fused_tiled<T, R, kFusedModes>(p, s) : run_fused<T, R, kFusedModes>(p, s);
 }
 
 template <typename T>
-cudaError_t fused_as(const StoreView &sv, const FactorSet &fs, int R, const HotRows *hot, float *const *outs,
-                     cudaStream_t s) {
+cudaError_t fused_as(const StoreView &sv, const TileOrder *to, const FactorSet &fs, int R, const HotRows *hot,
+                     float *const *outs, cudaStream_t s) {
     if (sv.end <= sv.begin) return cudaSuccess;
     FusedParams p;
     memset(&p, 0, sizeof(p));
@@ -395,7 +512,12 @@ cudaError_t fused_as(const StoreView &sv, const FactorSet &fs, int R, const HotR
         p.log2nb[n] = -1;
         p.wacc_off[n] = wf;
         p.table_off[n] = tb;
-        if (sv.dims[n] <= budget) {
+        if (to) {
+            p.rank[n] = to->rank[n];
+            p.hot_rows[n] = hot[n].rows;
+            p.kw[n] = std::min(std::min(hot[n].count, kOrderCold), budget);
+            if (sv.dims[n] > sv.dims[p.order_mode]) p.order_mode = n;
+        } else if (sv.dims[n] <= budget) {
             p.hot_dense[n] = 1;
             p.kw[n] = (int)sv.dims[n];
         } else if (hot[n].rows && hot[n].count > 0) {
@@ -428,12 +550,12 @@ bool fused_supported(const StoreView &sv, int R) {
     return true;
 }
 
-cudaError_t launch_mttkrp_fused(const StoreView &sv, const FactorSet &fs, blco_dtype fdt, int R, const HotRows *hot,
-                                float *const *outs, cudaStream_t s) {
+cudaError_t launch_mttkrp_fused(const StoreView &sv, const TileOrder *to, const FactorSet &fs, blco_dtype fdt, int R,
+                                const HotRows *hot, float *const *outs, cudaStream_t s) {
     switch (fdt) {
-        case BLCO_F32: return fused_as<float>(sv, fs, R, hot, outs, s);
-        case BLCO_BF16: return fused_as<__nv_bfloat16>(sv, fs, R, hot, outs, s);
-        case BLCO_F16: return fused_as<__half>(sv, fs, R, hot, outs, s);
+        case BLCO_F32: return fused_as<float>(sv, to, fs, R, hot, outs, s);
+        case BLCO_BF16: return fused_as<__nv_bfloat16>(sv, to, fs, R, hot, outs, s);
+        case BLCO_F16: return fused_as<__half>(sv, to, fs, R, hot, outs, s);
         default: break;
     }
     return cudaErrorInvalidValue;

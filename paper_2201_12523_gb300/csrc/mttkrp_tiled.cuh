@@ -38,6 +38,7 @@
 #include <atomic>
 
 #include "mttkrp_kernels.cuh"
+#include "tile_stage.cuh"
 
 namespace blco {
 namespace {
@@ -88,18 +89,6 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 template <int NG>
 __host__ __device__ constexpr int inner_slots() {
     return NG > 0 ? NG - 1 : kMaxGather - 2;  // at most MAXN - 2 inner modes
-}
-
-// Staged ranks: every subgroup's P ranks are followed by one unused entry, so
-// that the subgroups of a warp, which read P entries apart, hit different
-// banks (without it every record read is a 4-way conflict).
-template <int P>
-__host__ __device__ constexpr int staged() {
-    return kTile + kTile / P;
-}
-template <int P>
-__device__ __forceinline__ uint32_t staged_at(uint32_t r) {
-    return r + r / P;
 }
 
 // Shared memory of a CTA: a record per rank, `words` further words per rank,

@@ -108,3 +108,25 @@ def test_tiled_f64_nonfinite_rows_are_summed_term_by_term():
         assert np.array_equal(np.isnan(got), np.isnan(ref))
         assert np.array_equal(np.isposinf(got), np.isposinf(ref))
         assert np.array_equal(np.isneginf(got), np.isneginf(ref))
+
+
+@pytest.mark.parametrize("dims,nnz,line,R,dtype,skip", [
+    ((900, 800, 70, 60, 5), 65_536, 64, 16, torch.float32, None),
+    ((900, 800, 70, 60, 5), 65_537, 20, 32, torch.float32, None),    # blocks; one nonzero in the last tile
+    ((60, 70, 5000, 8, 9), 66_559, 64, 64, torch.float32, 2),       # the longest mode in the middle, not asked for
+    ((90, 80, 70, 60, 1), 70_001, 64, 16, torch.bfloat16, None),    # a mode of one row
+    ((1 << 24, 300, 20, 12, 10), 70_003, 40, 32, torch.float16, 1),  # the longest mode the kernel takes
+])
+def test_tiled_all_modes_in_one_pass(dims, nnz, line, R, dtype, skip):
+    rng, c = _coo(dims, nnz, nnz + R)
+    vals = rng.standard_normal(nnz).astype(np.float32)
+    t = blco.Tensor.build(_i32(c), torch.from_numpy(vals).cuda(), dims, line_bits=line)
+    A = [torch.from_numpy(rng.standard_normal((d, R)).astype(np.float32)).cuda().to(dtype) for d in dims]
+    outs = [None if n == skip else torch.full((d, R), 3.0, device="cuda") for n, d in enumerate(dims)]
+    blco.blco_mttkrp_all(t.handle, A, blco._DTYPE_CODE[dtype], R, outs)
+    Af = [a.double().cpu().numpy() for a in A]
+    for n in range(5):
+        if n == skip:
+            continue
+        M, S = oracle.mttkrp(c, vals.astype(np.float64), dims, Af, n)
+        assert oracle.max_rel_err(outs[n].cpu().numpy(), M, S) <= FP32_TOL
