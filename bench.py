@@ -60,8 +60,8 @@ FALLBACK_HBM_GBS = 6800.0
 FP32_TOL, BF16_TOL = 1e-5, 1e-2
 
 # DRAM traffic of the MTTKRP kernel per launch from one ncu capture
-# (profiles/), valid only for the kernel source it was taken from (sha256 of
-# the kernel header and its float32 translation unit): workload -> record.
+# (profiles/), valid only for the kernel source it was taken from (sha256, see
+# mttkrp_src_sha): workload -> record.
 TRAFFIC_RECORDS = {
     "zipf1.1-4d-500M": {"src_sha256": "e6765c8922a7d71eafc404c1d1ce06398280425ae954f857e53e8aeec58b933b",
                         "bytes_per_launch": 7.223e9},  # mean of modes 0-3, R = 32, float32 factors
@@ -198,11 +198,12 @@ def hbm_peak():
 
 
 def mttkrp_src_sha(onepass: bool = False) -> str:
-    """sha256 over the MTTKRP kernel's sources (the kernel header and the
-    float32 translation unit, or the one-pass kernel's unit), to tell whether
-    a recorded ncu traffic figure still describes the kernel being timed."""
+    """sha256 over the sources of the MTTKRP kernel of a resident store (the
+    kernel headers and the order of its tiles, with the one-pass kernel's unit
+    where that runs), to tell whether a recorded ncu traffic figure still
+    describes the kernel being timed."""
     h = hashlib.sha256()
-    for name in ("mttkrp_kernels.cuh", "mttkrp_fused.cu" if onepass else "mttkrp_f32.cu"):
+    for name in ("mttkrp_kernels.cuh", "tile_order.cu", "mttkrp_fused.cu" if onepass else "mttkrp_tiled.cuh"):
         with open(os.path.join(ROOT, "paper_2201_12523_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
@@ -479,11 +480,11 @@ def measure_mttkrp(blco, spec, args, ranks, dev, steps, warmup, *, headline, sam
     if onepass:
         b32 = onepass_bytes(spec, R, 4)
         touched_bytes = onepass_bytes(spec, R, 4, touched)
-        kname = f"k_mttkrp_fused<float,{R},{spec.order}>"
+        kname = f"k_mttkrp_fused_tiled<float,{R},{spec.order}>"
     else:
         b32 = sum(algorithmic_bytes(spec, R, 4, n) for n in range(spec.order)) / spec.order
         touched_bytes = sum(algorithmic_bytes(spec, R, 4, n, touched) for n in range(spec.order)) / spec.order
-        kname = f"k_mttkrp<float,{R},{spec.order - 1}>"
+        kname = f"k_mttkrp_tiled<float,{R},{spec.order - 1}>"
     ach, kms, kl = kernel_roofline(prof, kind, b32, peak)
     rec = TRAFFIC_RECORDS.get(spec.name)
     traffic = rec["bytes_per_launch"] if rec and rec["src_sha256"] == mttkrp_src_sha(onepass) else None
@@ -502,7 +503,7 @@ def measure_mttkrp(blco, spec, args, ranks, dev, steps, warmup, *, headline, sam
     res["clocks"] = clocks
     res["construction"] = {"ms": build_ms, "nnz_per_s": spec.nnz / (build_ms / 1e3),
                            "all_mode_steps_to_amortize": build_ms / res["ms_per_step"],
-                           "note": "blco_build from device coordinates: linearize, radix sort, block, re-encode, "
+                           "note": "blco_build from device coordinates: linearize, radix sort, block, re-encode, tile order, "
                                    "hot-row histograms" + (", move to pinned host memory" if info["streamed"] else "")}
     res["store"] = {"nblocks": info["nblocks"], "streamed": info["streamed"], "hot_rows": info["hot_rows"],
                     "device_bytes": info["device_bytes"], "host_bytes": info["host_bytes"]}

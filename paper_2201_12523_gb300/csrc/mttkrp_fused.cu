@@ -14,18 +14,20 @@
 // same. Where a mode's row changes, the run's sum goes to the warp's
 // shared-memory copy of the row if the row is one of that mode's hottest
 // (picked at build time), else to global memory with red.global.add.v4.f32.
-// Two subgroups may store the same hot row in the same step, so stores to
-// the shared copies are serialized over the subgroups that have one pending
-// (a warp ballot). Row ids and the row's slot in the shared copies are staged
-// as one word: id | slot << 24 (modes of at most 2^24 rows; slot 0xFF: no
-// copy).
+// Two subgroups may store the same hot row in the same step: every subgroup
+// with one pending claims it (a shared word per copied row), the claim that
+// stands updates the copy, the others claim again. Row ids and the row's slot
+// in the shared copies are staged as one word: id | slot << 24 (modes of at
+// most 2^24 rows; slot 0xFF: no copy).
 //
-// Without the per-mode sort a run ends at almost every nonzero, so each
-// nonzero costs N global or shared stores: the store side, not the gathers,
-// bounds this kernel. It pays where gathers dominate the per-mode kernels:
-// at 5 modes it runs 1.4-1.7x faster than five per-mode launches; at 3 and 4
-// modes the per-mode kernels (sorted tiles, 2 or 3 gathers per nonzero) are
-// as fast or faster, and blco_mttkrp_all uses them there.
+// Without a sort per mode a run ends at almost every nonzero, so each nonzero
+// costs N global or shared stores: the store side, not the gathers, bounds
+// this kernel. It pays where gathers dominate the per-mode kernels: on 50M
+// nonzeros of the 5-mode Zipf shape at R = 16 it takes 4.62 ms and, over the
+// order inside tiles (k_mttkrp_fused_tiled), 3.89, against 5.55 for five
+// launches of k_mttkrp_tiled; at 3 and 4 modes the per-mode kernels are as fast
+// or faster, and blco_mttkrp_all uses them there. Updating the copies one
+// subgroup after the other instead of by claims: 4.71.
 #include <algorithm>
 
 #include "mttkrp_kernels.cuh"
@@ -387,7 +389,9 @@ __global__ void __launch_bounds__(kThreads, fused_min_ctas<T, R, N>()) k_mttkrp_
 // row, so that this mode's runs and, inside them, those of the others last
 // longer than in store order, and a subgroup walks R ranks instead of R / 4
 // positions. Slots come with the ranks: no tables. 100M nonzeros of the 5-mode
-// Zipf shape, R = 16: 8.95 -> @FT@ ms.
+// Zipf shape, R = 16: 8.93 -> 7.28 ms. At 3 and
+// 4 modes (50M nonzeros) it is slower than the per-mode kernels from R = 32 on
+// (3.42 against 2.67 ms, 5.18 against 4.53) and equal at R = 16.
 template <typename T, int R, int N>
 __global__ void __launch_bounds__(kThreads, 2) k_mttkrp_fused_tiled(const FusedParams p) {
     constexpr int VEC = lane_vec<T, R>();
