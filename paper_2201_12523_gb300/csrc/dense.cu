@@ -64,11 +64,12 @@ __device__ __forceinline__ float to_f<__half>(__half v) { return __half2float(v)
 // Bound by the ten float32 operations per product. CTAs are as wide as whole
 // thread groups need (at most kGramThreads): with 256 threads, R = 64 left one
 // group of 136 threads and the other 120 idle, and 2^20 rows took 1.30 ms; two
-// groups in 288 threads take 1.09 (packed f32x2 arithmetic: 1.18, that pipe's
-// rate; two CTAs per SM without the register limit: 1.02, but 7-10 % slower at
-// R = 16 and 50).
+// groups in 288 threads take 1.02 with two CTAs per SM (1.13 with three, whose
+// 72 registers spill; at R = 16 and 50 three are 7-10 % faster, so two only
+// from kGramWideRank on). Packed f32x2 arithmetic: 1.18, that pipe's rate.
 constexpr int kGramRows = 32;  // rows staged in shared memory per step
 constexpr int kGramThreads = 288;
+constexpr int kGramWideRank = 60;
 
 struct GramShape {
     int R4;      // R rounded up to 4 (padding columns are zero)
@@ -118,8 +119,8 @@ __device__ __forceinline__ float inv_norm(double colsq, double *lambda) {
 // by their norms, in place, and the Gram is that of the scaled A; CTA 0 writes
 // lambda. Scaling here instead of in a pass of its own saves that pass's read
 // and write (0.15 ms at 2^20 x 64).
-template <typename T, bool SCALE>
-__global__ void __launch_bounds__(kGramThreads, 3) k_gram(const T *A, T *A_out, int64_t I, int R, int64_t rows_per_cta,
+template <typename T, bool SCALE, int CTAS>
+__global__ void __launch_bounds__(kGramThreads, CTAS) k_gram(const T *A, T *A_out, int64_t I, int R, int64_t rows_per_cta,
                                                        const double *__restrict__ colsq, double *__restrict__ lambda,
                                                        double *__restrict__ G) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -708,11 +709,12 @@ struct GramLaunch {
     int64_t rows;
 };
 
-// three CTAs per SM in total (the register limit), each over a contiguous
-// range of rows
+int gram_ctas(int R) { return R >= kGramWideRank ? 2 : 3; }
+
+// as many CTAs as are resident in total, each over a contiguous range of rows
 GramLaunch gram_launch(int64_t I, int R) {
     const GramShape sh = gram_shape(R);
-    const int64_t ctas_max = std::max<int64_t>(1, (int64_t)sm_count() * 3 / sh.ny);
+    const int64_t ctas_max = std::max<int64_t>(1, (int64_t)sm_count() * gram_ctas(R) / sh.ny);
     GramLaunch g;
     g.rows = (I + ctas_max - 1) / ctas_max;
     g.rows = std::max<int64_t>(kGramRows, (g.rows + kGramRows - 1) / kGramRows * kGramRows);
@@ -722,14 +724,23 @@ GramLaunch gram_launch(int64_t I, int R) {
     return g;
 }
 
-template <typename T>
-cudaError_t run_gram(const void *A, int64_t I, int R, double *G, cudaStream_t s) {
+template <typename T, bool SCALE, int CTAS>
+cudaError_t run_gram_as(const T *A, T *A_out, int64_t I, int R, const double *colsq, double *lambda, double *G,
+                        cudaStream_t s) {
     const GramLaunch g = gram_launch(I, R);
-    cudaError_t e = cudaFuncSetAttribute(k_gram<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.shm);
+    auto kern = k_gram<T, SCALE, CTAS>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.shm);
     if (e != cudaSuccess) return e;
-    k_gram<T, false><<<g.grid, g.threads, g.shm, s>>>(static_cast<const T *>(A), nullptr, I, R, g.rows, nullptr,
-                                                      nullptr, G);
+    kern<<<g.grid, g.threads, g.shm, s>>>(A, A_out, I, R, g.rows, colsq, lambda, G);
     return cudaGetLastError();
+}
+
+template <typename T, bool SCALE>
+cudaError_t run_gram(const void *A, T *A_out, int64_t I, int R, const double *colsq, double *lambda, double *G,
+                     cudaStream_t s) {
+    const T *a = static_cast<const T *>(A);
+    return gram_ctas(R) == 2 ? run_gram_as<T, SCALE, 2>(a, A_out, I, R, colsq, lambda, G, s)
+                             : run_gram_as<T, SCALE, 3>(a, A_out, I, R, colsq, lambda, G, s);
 }
 
 __global__ void k_zero_lambda(double *lambda, double *G, int R) {
@@ -761,11 +772,7 @@ cudaError_t run_update(const double *const *grams, int N, int mode, int R, const
     k_apply<<<(unsigned)ctas, kApplyThreads, shm, s>>>(M, I, R, Wf, A, colsq, G_out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const GramLaunch g = gram_launch(I, R);
-    e = cudaFuncSetAttribute(k_gram<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.shm);
-    if (e != cudaSuccess) return e;
-    k_gram<float, true><<<g.grid, g.threads, g.shm, s>>>(A, A, I, R, g.rows, colsq, lambda, G_out);
-    return cudaGetLastError();
+    return run_gram<float, true>(A, A, I, R, colsq, lambda, G_out, s);
 }
 
 }  // namespace
@@ -775,9 +782,9 @@ cudaError_t launch_gram(const void *A, blco_dtype fdt, int64_t I, int R, double 
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || I <= 0) return e;
     switch (fdt) {
-        case BLCO_F32: return run_gram<float>(A, I, R, G, s);
-        case BLCO_BF16: return run_gram<__nv_bfloat16>(A, I, R, G, s);
-        case BLCO_F16: return run_gram<__half>(A, I, R, G, s);
+        case BLCO_F32: return run_gram<float, false>(A, nullptr, I, R, nullptr, nullptr, G, s);
+        case BLCO_BF16: return run_gram<__nv_bfloat16, false>(A, nullptr, I, R, nullptr, nullptr, G, s);
+        case BLCO_F16: return run_gram<__half, false>(A, nullptr, I, R, nullptr, nullptr, G, s);
     }
     return cudaErrorInvalidValue;
 }
