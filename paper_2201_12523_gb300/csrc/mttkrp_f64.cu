@@ -64,21 +64,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_mttkrp64(const KParams p, const
     const int ng = n_gather<NG>(p);
 
     for (int i = threadIdx.x; i < kWarps * (kw + 1) * R; i += kThreads) wacc_all[i] = 0.0;
-    for (int i = threadIdx.x; i < nb; i += kThreads) table[i] = make_uint4(kNoRow, 0u, kNoRow, 0u);
-    __syncthreads();
-    if (nb > 0 && threadIdx.x == 0) {
-        for (int i = 0; i < kw; ++i) {
-            const uint32_t row = __ldg(p.hot_rows + i);
-            uint4 &bk = table[hot_hash(row, p.log2nb)];
-            if (bk.x == kNoRow) {
-                bk.x = row;
-                bk.y = (uint32_t)i;
-            } else if (bk.z == kNoRow) {
-                bk.z = row;
-                bk.w = (uint32_t)i;
-            }
-        }
-    }
+    if (nb > 0) fill_hot_table<kThreads>(table, nb, p.log2nb, p.hot_rows, kw, reinterpret_cast<uint32_t *>(smem));
     __syncthreads();
 
     const int64_t ntiles = (p.end - p.begin + 31) >> 5;

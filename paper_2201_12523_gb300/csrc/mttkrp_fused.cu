@@ -294,25 +294,13 @@ __global__ void __launch_bounds__(kThreads, fused_min_ctas<T, R, N>()) k_mttkrp_
     uint32_t *claim = reinterpret_cast<uint32_t *>(smem + L.claim) + wid * (p.warp_floats / R);
     uint4 *tables = reinterpret_cast<uint4 *>(smem + L.table);
 
-    // --- zero the copies; thread n fills mode n's table in order of decreasing count
+    // --- zero the copies, fill the modes' tables (the tiles' staging is scratch here)
     for (int i = threadIdx.x; i < kWarps * p.warp_floats; i += kThreads) wacc_all[i] = 0.f;
-    for (int i = threadIdx.x; i < p.table_buckets; i += kThreads) tables[i] = make_uint4(kNoRow, 0u, kNoRow, 0u);
-    __syncthreads();
-    if (threadIdx.x < N && p.log2nb[threadIdx.x] >= 0) {
-        const int n = threadIdx.x;
-        uint4 *tb = tables + p.table_off[n];
-        for (int i = 0; i < p.kw[n]; ++i) {
-            const uint32_t row = __ldg(p.hot_rows[n] + i);
-            uint4 &bk = tb[hot_hash(row, p.log2nb[n])];
-            if (bk.x == kNoRow) {
-                bk.x = row;
-                bk.y = (uint32_t)i;
-            } else if (bk.z == kNoRow) {
-                bk.z = row;
-                bk.w = (uint32_t)i;
-            }
-        }
-    }
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+        if (p.log2nb[n] >= 0)
+            fill_hot_table<kThreads>(tables + p.table_off[n], 1 << p.log2nb[n], p.log2nb[n], p.hot_rows[n], p.kw[n],
+                                     reinterpret_cast<uint32_t *>(smem));
     __syncthreads();
 
     const char *rowp[N];

@@ -353,25 +353,12 @@ __global__ void __launch_bounds__(kThreads, mttkrp_min_ctas<R, NG>()) k_mttkrp(c
     const int ng = n_gather<NG>(p);
     float *const outp = p.out + (p.ncopies > 1 ? (size_t)(blockIdx.x % p.ncopies) * p.copy_stride : 0);
 
-    // --- zero the accumulators; thread 0 fills the hot-row table in order of
-    // decreasing count (one hash, buckets of two (row, slot) pairs; a row that
-    // finds its bucket full stays off chip and is simply a cold row)
+    // --- zero the accumulators, fill the hot-row table (a row that finds its
+    // bucket full stays off chip and is simply a cold row; the tiles' staging
+    // is scratch here). One thread filling it took a load's latency per row:
+    // 10 us at the start of every launch with 32 rows.
     for (int i = threadIdx.x; i < kWarps * (kw + 1) * R; i += kThreads) wacc_all[i] = 0.f;
-    for (int i = threadIdx.x; i < nb; i += kThreads) table[i] = make_uint4(kNoRow, 0u, kNoRow, 0u);
-    __syncthreads();
-    if (nb > 0 && threadIdx.x == 0) {
-        for (int i = 0; i < kw; ++i) {
-            const uint32_t row = __ldg(p.hot_rows + i);
-            uint4 &bk = table[hot_hash(row, p.log2nb)];
-            if (bk.x == kNoRow) {
-                bk.x = row;
-                bk.y = (uint32_t)i;
-            } else if (bk.z == kNoRow) {
-                bk.z = row;
-                bk.w = (uint32_t)i;
-            }
-        }
-    }
+    if (nb > 0) fill_hot_table<kThreads>(table, nb, p.log2nb, p.hot_rows, kw, reinterpret_cast<uint32_t *>(smem));
     __syncthreads();
 
     const int64_t ntiles = (p.end - p.begin + 31) >> 5;
