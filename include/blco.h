@@ -115,7 +115,9 @@ typedef struct {
     int32_t hot_rows[BLCO_MAX_MODES];      /* hottest rows kept per mode (a launch at rank R
                                               accumulates the first min(this, 1024 / R)
                                               of them on chip) */
-    int64_t device_bytes;                  /* device memory held by the handle */
+    int64_t device_bytes;                  /* device memory held by the handle (with the
+                                              order inside tiles of a resident store:
+                                              about 2.1 bytes per nonzero and mode) */
     int64_t host_bytes;                    /* pinned host memory held by the handle */
     int32_t host_reads;                    /* 1 if kernels read the streamed store in host memory */
 } blco_info_t;
@@ -305,7 +307,7 @@ blco_status blco_gram(const void *A, blco_dtype fdt, int64_t I, int R, double *G
  *   lambda  R float64 output (device): the column norms removed from A
  *   G_out   R x R float64 output (device): Gram of the new A (may be NULL)
  *   info    1 int32 (device): 0 if every Cholesky pivot of V exceeded
- *           R * eps * max_i V_ii (Cholesky solve), 1 otherwise (V numerically
+ *           R * eps * max_i V_ii (inverse), 1 otherwise (V numerically
  *           singular or indefinite: the eigen pseudo-inverse, eigenvalues
  *           with |w| <= max|w| * R * eps dropped)
  * R in 1..64; larger ranks return BLCO_ERR_UNSUPPORTED.
