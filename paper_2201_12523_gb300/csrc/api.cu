@@ -36,6 +36,8 @@ constexpr int64_t kDefaultCap = (int64_t)1 << 27;
 // nonzeros 14-19 us against 19-24, 600k 18-25 against 25-41; at 64k a launch is
 // mostly latency either way (64 tiles).
 constexpr int64_t kOrderMinNnz = (int64_t)1 << 16;
+// Modes for which a float64 store keeps it: those k_mttkrp64_tiled is faster at.
+bool order_pays_f64(int N) { return N == 3 || N == 4; }
 
 blco_status fail(blco_status st, const std::string &msg) {
     g_err = msg;
@@ -746,7 +748,8 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
     // The order inside tiles: for stores without a device budget (which is the
     // caller's to divide) that have it in a quarter of the free memory. A store
     // without it is served by the kernels that order 32 nonzeros at a time.
-    if (!h->streamed && h->budget == 0 && tile_order_supported(h->L) && nnz >= kOrderMinNnz) {
+    if (!h->streamed && h->budget == 0 && tile_order_supported(h->L) && nnz >= kOrderMinNnz &&
+        (!no_vals || order_pays_f64(N))) {
         const size_t ob = tile_order_bytes(nnz, N, no_vals);
         size_t free_b = 0, total_b = 0;
         if ((ob <= ((size_t)16 << 20) || (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && ob <= free_b / 4)) &&

@@ -334,7 +334,11 @@ __global__ void __launch_bounds__(kTiledThreads, tiled_min_ctas<R, NG>()) k_mttk
 // gathered row and a sum are N operations per nonzero. A subgroup is a whole
 // warp from R = 32 on, so a fiber's end costs only the warp that has one. 20M
 // nonzeros of the 3-mode Zipf shape (2^20, 2^19, 2^11), R = 32, all modes:
-// 10.9 ms with the kernel of mttkrp_f64.cu, 6.8 here.
+// 10.9 ms with the kernel of mttkrp_f64.cu, 6.8 here. For 3 and 4 modes
+// (order_pays_f64): without an inner mode a fiber's sum takes as many
+// operations as the terms, and from 5 modes on fibers are one or two nonzeros
+// long (2 modes 10M nonzeros, R = 32: 2.7 ms there, 8.7 here; 5 modes 2M, R =
+// 64: 6.3 and 10.6; 7 modes 10M, R = 32: 0.90 of its speed).
 __device__ __forceinline__ void red_add_double(double *addr, double v) {
     asm volatile("red.global.add.f64 [%0], %1;" ::"l"(addr), "d"(v));
 }
@@ -364,11 +368,10 @@ __device__ __forceinline__ bool is_finite(double x) {
 // product is not the sum of the terms (0 times infinity among them).
 template <int NI>
 __device__ __noinline__ double add_terms(double acc, const Rec64 *rp, const uint32_t *xp, int stride, int n,
-                                         const TParams &p, int ni, int R, int e, double k) {
+                                         const TParams &p, int R, int e, double k) {
     for (int r = 0; r < n; ++r) {
-        double x = rp[r].val;
-        if (ni > 0) x *= __ldg(static_cast<const double *>(p.gat[0].ptr) + (size_t)rp[r].in * R + e);
-        for (int q = 1; q < ni; ++q)
+        double x = rp[r].val * __ldg(static_cast<const double *>(p.gat[0].ptr) + (size_t)rp[r].in * R + e);
+        for (int q = 1; q < NI; ++q)
             x *= __ldg(static_cast<const double *>(p.gat[q].ptr) + (size_t)xp[(q - 1) * stride + r] * R + e);
         acc = fma(x, k, acc);
     }
@@ -376,7 +379,7 @@ __device__ __noinline__ double add_terms(double acc, const Rec64 *rp, const uint
 }
 
 template <int R, int NG>
-__global__ void __launch_bounds__(kTiledThreads, R > 32 || NG == 0 ? 2 : 3) k_mttkrp64_tiled(const TParams p) {
+__global__ void __launch_bounds__(kTiledThreads, R > 32 ? 2 : 3) k_mttkrp64_tiled(const TParams p) {
     constexpr int G = R < 32 ? R : 32;
     constexpr int VEC = R / G;
     constexpr int SUBS = kTiledThreads / G;
@@ -384,11 +387,11 @@ __global__ void __launch_bounds__(kTiledThreads, R > 32 || NG == 0 ? 2 : 3) k_mt
     constexpr int CH = 4;
     constexpr int NI = inner_slots<NG>();
     static_assert(P % 32 == 0 && VEC <= 2, "whole words of the bit masks");
+    static_assert(NG == 2 || NG == 3, "one or two inner modes");
 
     extern __shared__ __align__(16) unsigned char smem[];
-    const int ni = NG > 0 ? NG - 1 : p.n_inner;
     // one word per rank more than the float32 kernel: the target row or slot
-    const TiledSmem L = tiled_smem(sizeof(Rec64), staged<P>(), (ni > 1 ? ni - 1 : 0) + 1, p.kw, R * sizeof(double));
+    const TiledSmem L = tiled_smem(sizeof(Rec64), staged<P>(), NI, p.kw, R * sizeof(double));
     Rec64 *rec = reinterpret_cast<Rec64 *>(smem);
     uint32_t *srow = reinterpret_cast<uint32_t *>(smem + L.extra);
     uint32_t *extra = srow + staged<P>();
@@ -413,7 +416,7 @@ __global__ void __launch_bounds__(kTiledThreads, R > 32 || NG == 0 ? 2 : 3) k_mt
         uint32_t ew = __ldg(endw), fw = __ldg(fendw);
         prefetch_tile(p, tile + gridDim.x, ntiles, p.vals64, (int)sizeof(double));
         stage_tile<NI, P>(
-            p, base, nvalid, ni,
+            p, base, nvalid, NI,
             [&](uint32_t r, bool valid, int q, uint32_t o, uint32_t k, uint32_t row) {
                 Rec64 rc;
                 rc.val = valid ? __ldcs(p.vals64 + base + q) : 0.0;
@@ -452,29 +455,27 @@ __global__ void __launch_bounds__(kTiledThreads, R > 32 || NG == 0 ? 2 : 3) k_mt
                     for (int j = 0; j < CH; ++j) rc[j] = rp[j];
 #pragma unroll
                     for (int j = 0; j < CH; ++j)
-                        if (NG != 0 || ni > 0) load_doubles<VEC>(inp + (size_t)rc[j].in * R, x[j]);
+                        load_doubles<VEC>(inp + (size_t)rc[j].in * R, x[j]);
 #pragma unroll
                     for (int j = 0; j < CH; ++j)
                         if (fe & (1u << j)) load_doubles<VEC>(parp + (size_t)rc[j].par * R, k[j]);
 #pragma unroll
                     for (int q = 1; q < NI; ++q) {
-                        if (q < ni) {
-                            const double *gp = static_cast<const double *>(p.gat[q].ptr) + c * VEC;
-                            double g[CH][VEC];
+                        const double *gp = static_cast<const double *>(p.gat[q].ptr) + c * VEC;
+                        double g[CH][VEC];
 #pragma unroll
-                            for (int j = 0; j < CH; ++j)
-                                load_doubles<VEC>(gp + (size_t)xp[(q - 1) * staged<P>() + j] * R, g[j]);
+                        for (int j = 0; j < CH; ++j)
+                            load_doubles<VEC>(gp + (size_t)xp[(q - 1) * staged<P>() + j] * R, g[j]);
 #pragma unroll
-                            for (int j = 0; j < CH; ++j)
+                        for (int j = 0; j < CH; ++j)
 #pragma unroll
-                                for (int i = 0; i < VEC; ++i) x[j][i] *= g[j][i];
-                        }
+                            for (int i = 0; i < VEC; ++i) x[j][i] *= g[j][i];
                     }
 #pragma unroll
                     for (int j = 0; j < CH; ++j) {
 #pragma unroll
                         for (int i = 0; i < VEC; ++i)
-                            fs[i] = (NG != 0 || ni > 0) ? fma(rc[j].val, x[j][i], fs[i]) : fs[i] + rc[j].val;
+                            fs[i] = fma(rc[j].val, x[j][i], fs[i]);
                         if (fe & (1u << j)) {
 #pragma unroll
                             for (int i = 0; i < VEC; ++i) {
@@ -482,7 +483,7 @@ __global__ void __launch_bounds__(kTiledThreads, R > 32 || NG == 0 ? 2 : 3) k_mt
                                     acc[i] = fma(fs[i], k[j][i], acc[i]);
                                 else
                                     acc[i] = add_terms<NI>(acc[i], rec + first, extra + first, staged<P>(),
-                                                           (int)(rp + j - rec) - first + 1, p, ni, R, c * VEC + i,
+                                                           (int)(rp + j - rec) - first + 1, p, R, c * VEC + i,
                                                            k[j][i]);
                                 fs[i] = 0.0;
                             }
@@ -650,8 +651,7 @@ cudaError_t run_tiled64(const TParams &p, cudaStream_t s) {
     static std::atomic<uint64_t> last{0};
     return launch_tiled(
         k_mttkrp64_tiled<R, NG>, p,
-        tiled_smem(sizeof(Rec64), staged<P>(), (p.n_inner > 1 ? p.n_inner - 1 : 0) + 1, p.kw, R * sizeof(double)).total,
-        last, s);
+        tiled_smem(sizeof(Rec64), staged<P>(), inner_slots<NG>(), p.kw, R * sizeof(double)).total, last, s);
 }
 
 template <int R>
@@ -659,8 +659,8 @@ cudaError_t tiled64_by_ng(const TParams &p, cudaStream_t s) {
     switch (p.n_inner) {
         case 1: return run_tiled64<R, 2>(p, s);
         case 2: return run_tiled64<R, 3>(p, s);
-        default: return run_tiled64<R, 0>(p, s);
     }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace

@@ -1,0 +1,36 @@
+"""Which stores keep the order inside tiles of 1024 positions: those whose calls
+are faster with it. A store built with a device budget never keeps it, so the
+difference of the two stores' device memory is the order's."""
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+blco = pytest.importorskip("paper_2201_12523_gb300.blco")
+
+
+def _order_bytes(dims, nnz, dtype):
+    rng = np.random.default_rng(nnz)
+    c = np.stack([rng.integers(0, d, nnz) for d in dims], 1).astype(np.uint32).view(np.int32)
+    coords, vals = torch.from_numpy(np.ascontiguousarray(c)).cuda(), torch.ones(nnz, dtype=dtype, device="cuda")
+    plain = blco.Tensor.build(coords, vals, dims)
+    bare = blco.Tensor.build(coords, vals, dims, device_budget_bytes=1 << 33)
+    n = blco.blco_info(plain.handle).device_bytes - blco.blco_info(bare.handle).device_bytes
+    plain.destroy()
+    bare.destroy()
+    return n
+
+
+# per mode and tile: a 2-byte word per position, a bit per position, and in
+# float64 stores a second one
+def _expected(order, nnz, f64):
+    return order * -(-nnz // 1024) * (2048 + 128 * (2 if f64 else 1))
+
+
+@pytest.mark.parametrize("order,kept", [(1, False), (2, False), (3, True), (4, True), (5, False), (6, False), (8, False)])
+def test_float64_stores_keep_the_order_for_3_and_4_modes(order, kept):
+    nnz = 600_001
+    got = _order_bytes((3000, 700, 300, 90, 40, 9, 5, 3)[:order], nnz, torch.float64)
+    assert got == (_expected(order, nnz, True) if kept else 0)
