@@ -31,11 +31,19 @@ int sm_count() {
 namespace {
 
 constexpr int64_t kDefaultCap = (int64_t)1 << 27;
-// Fewest nonzeros for which the order inside tiles is kept. Measured on one
-// MTTKRP (host call included; tile order against 32 at a time, R = 32): 300k
-// nonzeros 14-19 us against 19-24, 600k 18-25 against 25-41; at 64k a launch is
-// mostly latency either way (64 tiles).
-constexpr int64_t kOrderMinNnz = (int64_t)1 << 16;
+// Fewest nonzeros for which the order inside tiles is kept, and from which calls
+// at R <= 64 use it. A launch has a CTA per tile of 1024: below two rounds of
+// them over the SMs (1.2M nonzeros at 4 CTAs per SM) the kernels that order 32
+// nonzeros at a time spread the work better. Speed with the order over without,
+// sums over modes of random shapes of 2 to 8 modes, uniform and Zipf:
+//   float32 and 16-bit, R <= 64: 66k 0.36-1.07, 200k 0.73-1.0, 500k 0.76-1.3,
+//     1.05M 0.93-1.5, 2M 0.95-1.45, 3M 1.0-2.1; one pass over 5 modes: 66k
+//     0.62-0.94, 500k 0.92-1.12, 1.05M 0.94-1.15, 5M 1.0-1.18;
+//   R = 128 (8 rows per launch on chip without the order): 66k 0.36-0.9, 200k
+//     0.73-1.1, 500k 0.76-1.3, from 700k 1.0-1.7;
+//   float64, 3 and 4 modes: 70k 0.6-1.0, 200k 0.8-1.3, 500k 0.82-1.46, 1M 1.1-1.5.
+constexpr int64_t kOrderMinNnz = (int64_t)1 << 19;
+constexpr int64_t kTiledMinNnz = (int64_t)1 << 20;
 // Modes for which a float64 store keeps it: those k_mttkrp64_tiled is faster at.
 bool order_pays_f64(int N) { return N == 3 || N == 4; }
 
@@ -454,6 +462,9 @@ HotRows hot_for(const blco_tensor *h, int mode, int R) {
     return hr;
 }
 
+// Whether a call at rank R over the whole store uses its order inside tiles.
+bool use_order(const blco_tensor *h, int R) { return h->d_order && (R > 64 || h->nnz >= kTiledMinNnz); }
+
 // The most frequent rows of `mode`, for kernels that choose how many they hold.
 HotRows hot_all(const blco_tensor *h, int mode) {
     HotRows hr;
@@ -499,7 +510,7 @@ blco_status mttkrp_device(blco_tensor *h, int mode, const FactorSet &fs, blco_dt
     cudaError_t e = cudaSuccess;
     if (!zeroed || dst != out) e = timed(h, "zero", s, [&]() { return launch_zero(dst, n * oc.n, s); });
     if (e != cudaSuccess) return cuda_fail(e, "zero output");
-    const bool tiled = h->d_order && range_end < 0 && !(h->compensated && fdt != BLCO_F32);
+    const bool tiled = use_order(h, R) && range_end < 0 && !(h->compensated && fdt != BLCO_F32);
     blco_status st = over_store(
         h, "mttkrp", vals_ext, s,
         [&](const StoreView &sv, cudaStream_t q) {
@@ -1067,7 +1078,7 @@ static blco_status mttkrp_all_onepass(blco_tensor *h, FactorSet fs, const bool *
         if (fused)
             return timed(h, "mttkrp_all_fused", q,
                          [&]() {
-                             return launch_mttkrp_fused(sv, h->d_order ? &h->order : nullptr, fs, fdt, R, hot_all,
+                             return launch_mttkrp_fused(sv, use_order(h, R) ? &h->order : nullptr, fs, fdt, R, hot_all,
                                                         dst_all, q);
                          });
         for (int n = 0; n < N; ++n) {

@@ -34,3 +34,12 @@ def test_float64_stores_keep_the_order_for_3_and_4_modes(order, kept):
     nnz = 600_001
     got = _order_bytes((3000, 700, 300, 90, 40, 9, 5, 3)[:order], nnz, torch.float64)
     assert got == (_expected(order, nnz, True) if kept else 0)
+
+
+@pytest.mark.parametrize("dtype,dims", [(torch.float32, (700, 90)), (torch.float32, (700, 300, 90, 40, 9)),
+                                        (torch.float64, (700, 300, 90))])
+def test_small_stores_keep_no_order(dtype, dims):
+    for nnz in (66_000, (1 << 19) - 1):
+        assert _order_bytes(dims, nnz, dtype) == 0
+    for nnz in (1 << 19, (1 << 19) + 1):
+        assert _order_bytes(dims, nnz, dtype) == _expected(len(dims), nnz, dtype == torch.float64)
