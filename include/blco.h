@@ -355,7 +355,8 @@ blco_status blco_cpals_fit(double normX2, const double *const *grams, int N, int
                            const double *lambda, const float *M_last, const float *A_last,
                            int64_t I_last, double *fit, blco_stream stream);
 
-/* sum_j vals[j]^2 in float64 over the stored values (device result). */
+/* sum_j vals[j]^2 over the stored values (device result), to the accuracy and
+ * over the range of a float64 sum. */
 blco_status blco_norm2(blco_handle h, double *out, blco_stream stream);
 
 /*

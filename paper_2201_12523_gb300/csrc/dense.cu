@@ -107,6 +107,43 @@ __device__ __forceinline__ void dot2_add(float x, float y, float &hi, float &lo)
     lo = __fadd_rn(lo, __fadd_rn(err, e));
 }
 
+// A sum of products in three floats, four terms at a time. The products and
+// the sum of the four are split free of error (TwoProduct, TwoSum), the small
+// parts of the four added in float32, and both added to the sum with their
+// errors kept (as Dot3 of Ogita, Rump and Oishi, 2005): 13 float32 operations a
+// term, where float64 takes a conversion and an FMA of a pipe with 2 lanes per
+// SM. For columns of 1 to 2^20 normal numbers the result (added over threads
+// and CTAs in float64) is off by at most 8e-16, the float64 sum it stands for
+// by 4e-15; Dot2, whose error grows with the terms of a thread, by 5e-13 at 500.
+// All that while the products are in float32's range: one is off by up to
+// 2^-149 where it or its error underflows, which 2^22 terms keep below 2^-53 of
+// a sum of 2^-70 or more, and not finite where it overflows. trusted() tells; a
+// thread whose sum is not takes it again in float64.
+struct WideSum {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(const float (&x)[4], const float (&y)[4]) {
+        float p[4], e[4], s0, s1, t, r0, r1, r2, a, b, c;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            p[i] = __fmul_rn(x[i], y[i]);
+            e[i] = __fmaf_rn(x[i], y[i], -p[i]);
+        }
+        two_sum(p[0], p[1], s0, r0);
+        two_sum(p[2], p[3], s1, r1);
+        two_sum(s0, s1, t, r2);
+        const float u = __fadd_rn(__fadd_rn(__fadd_rn(e[0], e[1]), __fadd_rn(e[2], e[3])),
+                                  __fadd_rn(__fadd_rn(r0, r1), r2));
+        two_sum(hi, t, hi, a);
+        two_sum(mid, u, mid, b);
+        two_sum(mid, a, mid, c);
+        lo = __fadd_rn(lo, __fadd_rn(b, c));
+    }
+    __device__ __forceinline__ bool trusted() const {
+        return fabsf(hi) >= 0x1p-70f && fabsf(hi) < INFINITY && fabsf(__fadd_rn(mid, lo)) < INFINITY;
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
+};
+
 // Column scales from the columns' sums of squares: lambda = sqrt, 1 / lambda
 // (1 for a zero column).
 __device__ __forceinline__ float inv_norm(double colsq, double *lambda) {
@@ -443,14 +480,15 @@ __global__ void __launch_bounds__(kSolveThreads) k_solve_small(const GramPtrs gp
     if (tid == 0) *info = 1;
 }
 
-// A = M W (float32) and the columns' sums of squares (Dot2, float64 between
+// A = M W (float32) and the columns' sums of squares (WideSum, float64 between
 // threads and CTAs). A thread computes 4 rows x 4 columns of a tile staged in
 // shared memory, summing over k in increasing order with one FMA per term; A
 // may be M. G, if not NULL, is zeroed for the Gram that follows.
 //
 // Bound by the float32 FMAs at R = 64 (2 I R^2), by HBM at small R. One warp
 // per row with two shared loads per FMA took 0.95 ms at 2^20 x 64 and a
-// float64 pass for the sums of squares 0.25; together 0.27 here.
+// float64 pass for the sums of squares 0.25; together 0.30 here, 0.03 of it the
+// sums (four CTAs per SM: at 74 registers, three, it took 0.04 more).
 constexpr int kApplyThreads = 256;
 
 struct ApplyShape {
@@ -474,7 +512,20 @@ inline size_t apply_smem(int R) {
     return std::max(stage, sizeof(double) * 4 * kApplyThreads);
 }
 
-__global__ void __launch_bounds__(kApplyThreads) k_apply(const float *M, int64_t I, int R,
+// Sum of squares in float64 of the entries of column `c` that a thread of row
+// group `rg` has stored. Apart, so that it costs k_apply no registers.
+__device__ __noinline__ double stored_squares(const float *A, int64_t I, int R, int c, int rg) {
+    const ApplyShape sh = apply_shape(R);
+    double v = 0.0;
+    for (int64_t i0 = (int64_t)blockIdx.x * sh.rows; i0 < I; i0 += (int64_t)gridDim.x * sh.rows)
+        for (int64_t i = i0 + rg; i < I && i < i0 + sh.rows; i += sh.rg) {
+            const double x = A[i * R + c];
+            v += x * x;
+        }
+    return v;
+}
+
+__global__ void __launch_bounds__(kApplyThreads, 4) k_apply(const float *M, int64_t I, int R,
                                                          const float *__restrict__ Wg, float *A,
                                                          double *__restrict__ colsq, double *__restrict__ G) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -490,9 +541,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply(const float *M, int64_t
         W[p] = k < R && n < R ? Wg[k * R + n] : 0.f;
     }
     const bool vec = R == sh.R4 && ((reinterpret_cast<uintptr_t>(M) | reinterpret_cast<uintptr_t>(A)) & 15) == 0;
-    float hi[4], lo[4];
-#pragma unroll
-    for (int n = 0; n < 4; ++n) hi[n] = lo[n] = 0.f;
+    WideSum sq[4];
     const int64_t ntiles = (I + sh.rows - 1) / sh.rows;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t i0 = t * sh.rows;
@@ -535,7 +584,11 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply(const float *M, int64_t
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             const int r = rg + a * sh.rg;
-            if (r >= nr) continue;
+            if (r >= nr) {
+#pragma unroll
+                for (int n = 0; n < 4; ++n) acc[a][n] = 0.f;
+                continue;
+            }
             float *dst = A + (i0 + r) * R + c;
             if (vec) {
                 *reinterpret_cast<float4 *>(dst) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
@@ -544,15 +597,21 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply(const float *M, int64_t
                 for (int n = 0; n < 4; ++n)
                     if (c + n < R) dst[n] = acc[a][n];
             }
+        }
 #pragma unroll
-            for (int n = 0; n < 4; ++n) dot2_add(acc[a][n], acc[a][n], hi[n], lo[n]);
+        for (int n = 0; n < 4; ++n) {
+            const float x[4] = {acc[0][n], acc[1][n], acc[2][n], acc[3][n]};
+            sq[n].add(x, x);
         }
     }
     __syncthreads();
     double *red = reinterpret_cast<double *>(smem);  // [rg][R4]
     if (rg < sh.rg)
 #pragma unroll
-        for (int n = 0; n < 4; ++n) red[rg * sh.R4 + c + n] = (double)hi[n] + (double)lo[n];
+        for (int n = 0; n < 4; ++n) {
+            red[rg * sh.R4 + c + n] =
+                c + n >= R || sq[n].trusted() ? sq[n].value() : stored_squares(A, I, R, c + n, rg);
+        }
     __syncthreads();
     if (tid < R) {
         double v = 0.0;
@@ -561,17 +620,37 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply(const float *M, int64_t
     }
 }
 
-// <M, A> per column (Dot2, float64 between threads and CTAs) -> acc[R]
+// <M, A> per column (WideSum, float64 between threads and CTAs) -> acc[R]
 __global__ void __launch_bounds__(256) k_coldot(const float *__restrict__ M, const float *__restrict__ A, int64_t I,
                                                 int R, double *__restrict__ acc) {
     __shared__ double red[256];
     const int nsub = 256 / R;
     const int c = threadIdx.x % R, sub = threadIdx.x / R;
-    float hi = 0.f, lo = 0.f;
-    if (sub < nsub)
-        for (int64_t i = (int64_t)blockIdx.x * nsub + sub; i < I; i += (int64_t)gridDim.x * nsub)
-            dot2_add(M[i * R + c], A[i * R + c], hi, lo);
-    red[threadIdx.x] = (double)hi + (double)lo;
+    double part = 0.0;
+    if (sub < nsub) {
+        const int64_t first = (int64_t)blockIdx.x * nsub + sub, step = (int64_t)gridDim.x * nsub;
+        WideSum d;
+        int64_t i = first;
+        for (; i + 3 * step < I; i += 4 * step) {
+            float x[4], y[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                x[k] = M[(i + k * step) * R + c];
+                y[k] = A[(i + k * step) * R + c];
+            }
+            d.add(x, y);
+        }
+        for (; i < I; i += step) {
+            const float x[4] = {M[i * R + c], 0.f, 0.f, 0.f}, y[4] = {A[i * R + c], 0.f, 0.f, 0.f};
+            d.add(x, y);
+        }
+        part = d.value();
+        if (!d.trusted()) {
+            part = 0.0;
+            for (int64_t i = first; i < I; i += step) part += (double)M[i * R + c] * (double)A[i * R + c];
+        }
+    }
+    red[threadIdx.x] = part;
     __syncthreads();
     if (threadIdx.x < R) {
         double v = 0.0;
@@ -612,14 +691,25 @@ __global__ void __launch_bounds__(256) k_fit_final(double normX2, const GramPtrs
     }
 }
 
-// Dot2 per thread, float64 between threads: bound by the read of v (in float64
+// WideSum per thread, float64 between threads: bound by the read of v (in float64
 // throughout, 8M values took 36 us; now 22).
 __global__ void __launch_bounds__(256) k_norm2(const float *__restrict__ v, int64_t n, double *__restrict__ out) {
-    float hi = 0.f, lo = 0.f;
-#pragma unroll 4
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dot2_add(v[i], v[i], hi, lo);
-    double s = (double)hi + (double)lo;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    WideSum d;
+    int64_t i = first;
+    for (; i + 3 * step < n; i += 4 * step) {
+        const float x[4] = {v[i], v[i + step], v[i + 2 * step], v[i + 3 * step]};
+        d.add(x, x);
+    }
+    for (; i < n; i += step) {
+        const float x[4] = {v[i], 0.f, 0.f, 0.f};
+        d.add(x, x);
+    }
+    double s = d.value();
+    if (!d.trusted()) {
+        s = 0.0;
+        for (int64_t i = first; i < n; i += step) s += (double)v[i] * (double)v[i];
+    }
     for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
 }
