@@ -1144,17 +1144,21 @@ blco_status blco_mttkrp_all(blco_handle h, const void *const *factors, blco_dtyp
         return mttkrp_all_onepass(h, fs, host_in, host_out, in_off, out_off, total, fdt, R, outs, s, fused);
     if (total == 0) {  // device arguments: the modes one after another on s
         // every output zeroed by one launch, unless one of them shares memory
-        // with a factor that an earlier mode still gathers
+        // with a factor that an earlier mode still gathers, or with another
+        // output (of which the later mode's result stands)
         int64_t len[MAXN] = {};
         bool apart = true;
         for (int n = 0; n < N; ++n) {
             if (!outs[n]) continue;
             len[n] = h->L.dims[n] * (int64_t)R;
             const uintptr_t o0 = reinterpret_cast<uintptr_t>(outs[n]), o1 = o0 + len[n] * sizeof(float);
-            for (int k = 0; k < N; ++k) {
-                const uintptr_t f0 = reinterpret_cast<uintptr_t>(factors[k]);
-                apart &= o1 <= f0 || f0 + h->L.dims[k] * (int64_t)R * dtype_size(fdt) <= o0;
-            }
+            const auto clear_of = [&](const void *a, size_t bytes) {
+                const uintptr_t a0 = reinterpret_cast<uintptr_t>(a);
+                return o1 <= a0 || a0 + bytes <= o0;
+            };
+            for (int k = 0; k < N; ++k) apart &= clear_of(factors[k], h->L.dims[k] * (int64_t)R * dtype_size(fdt));
+            for (int k = 0; k < n; ++k)
+                if (outs[k]) apart &= clear_of(outs[k], len[k] * sizeof(float));
         }
         if (apart) {
             cudaError_t e = timed(h, "zero", s, [&]() { return launch_zero_list(outs, len, N, s); });
