@@ -146,7 +146,8 @@ struct BuildOut {
     int64_t first_bad = -1;       // first coordinate row out of range
 };
 // Runs linearize / sort / re-encode / block on the device. coords and vals
-// are device pointers. Temporary memory via cudaMallocAsync on s.
+// are device pointers. Returns when its work on s is complete; waits for no other
+// stream.
 cudaError_t build_store(const Layout &L, const uint32_t *coords, const float *vals, int64_t nnz,
                         int64_t cap, BuildOut &out, cudaStream_t s, std::string &why);
 // dst[j] = src[perm[j]] for j < nnz (float64 values into store order)
