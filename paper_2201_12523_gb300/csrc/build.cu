@@ -388,7 +388,7 @@ cudaError_t radix_sort_pairs(K *keys, uint32_t *vals, K *kalt, uint32_t *valt, c
                              int nbits, uint32_t *counts, cudaStream_t s) {
     const int64_t ntiles = (n + kRsTile - 1) / kRsTile;
     const size_t shm = rs_scatter_smem<K>();
-    cudaError_t e = cudaFuncSetAttribute(k_rs_scatter<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    cudaError_t e = allow_smem((const void *)k_rs_scatter<K>, shm);
     const int passes = rs_passes(nbits);
     K *ki = key_source(keys, kalt, nbits);
     const uint32_t *vi = vals_in;
@@ -793,7 +793,7 @@ cudaError_t build_store(const Layout &L, const uint32_t *coords, const float *va
             uint64_t *src = key_source(out.keys, lo, (int)nbits);
             const size_t shm = (size_t)a.ntables * 256 * sizeof(uint64_t) * (wide ? 2 : 1);
             if (wide) {
-                TRY(cudaFuncSetAttribute(k_linearize<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+                TRY(allow_smem((const void *)k_linearize<true>, shm));
                 k_linearize<true><<<table_grid(nnz), 256, shm, s>>>(coords, nnz, a, src, hi, d_bad);
             } else {
                 k_linearize<false><<<table_grid(nnz), 256, shm, s>>>(coords, nnz, a, src, nullptr, d_bad);

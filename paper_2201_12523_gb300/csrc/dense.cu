@@ -819,7 +819,7 @@ cudaError_t run_gram_as(const T *A, T *A_out, int64_t I, int R, const double *co
                         cudaStream_t s) {
     const GramLaunch g = gram_launch(I, R);
     auto kern = k_gram<T, SCALE, CTAS>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.shm);
+    cudaError_t e = allow_smem((const void *)kern, g.shm);
     if (e != cudaSuccess) return e;
     kern<<<g.grid, g.threads, g.shm, s>>>(A, A_out, I, R, g.rows, colsq, lambda, G);
     return cudaGetLastError();
@@ -845,7 +845,7 @@ cudaError_t run_update(const double *const *grams, int N, int mode, int R, const
     GramPtrs gp;
     for (int k = 0; k < MAXN; ++k) gp.g[k] = k < N ? grams[k] : nullptr;
     const size_t shm_solve = sizeof(double) * 2 * R * R;
-    cudaError_t e = cudaFuncSetAttribute(k_solve_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_solve);
+    cudaError_t e = allow_smem((const void *)k_solve_small, shm_solve);
     if (e != cudaSuccess) return e;
     k_solve_small<<<1, kSolveThreads, shm_solve, s>>>(gp, N, mode, R, Wf, colsq, info);
     e = cudaGetLastError();
@@ -855,7 +855,7 @@ cudaError_t run_update(const double *const *grams, int N, int mode, int R, const
         return cudaGetLastError();
     }
     const size_t shm = apply_smem(R);
-    e = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    e = allow_smem((const void *)k_apply, shm);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (I + apply_shape(R).rows - 1) / apply_shape(R).rows;
     const int64_t ctas = std::min<int64_t>(tiles, (int64_t)sm_count() * 4);

@@ -37,6 +37,16 @@ struct Layout {
 // shape is unsupported (B > 128 or more than 64 block-key bits).
 bool plan_layout(Layout &L, std::string &why);
 
+// Lets a launch of `kern` use `shm` bytes of dynamic shared memory. Up to 46 KB
+// (48 with a kernel's static arrays) need no call; beyond that the limit is set
+// to the same value every time, so that a thread with another handle and size,
+// whose call may come between this one and its launch, does not lower it.
+inline cudaError_t allow_smem(const void *kern, size_t shm) {
+    constexpr size_t kFree = 46 * 1024;
+    constexpr int kLimit = 200 * 1024;  // more than any kernel here asks for
+    return shm <= kFree ? cudaSuccess : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kLimit);
+}
+
 // View of (part of) a store for one kernel launch.
 struct StoreView {
     const uint64_t *keys;   // in-block keys; keys[p - key_origin] for store position p

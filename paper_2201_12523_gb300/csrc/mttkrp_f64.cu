@@ -202,7 +202,7 @@ cudaError_t run_mttkrp64(const KParams &p, const double *vals64, double *out, cu
     const int nb = p.log2nb >= 0 ? (1 << p.log2nb) : 0;
     const size_t shm = smem_layout64(sizeof(Stage64<NG>), p.kw, R, nb).total;
     auto kern = k_mttkrp64<R, NG>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    cudaError_t e = allow_smem((const void *)kern, shm);
     if (e != cudaSuccess) return e;
     const int grid = grid_for((const void *)kern, shm, p.end - p.begin);
     kern<<<grid, kThreads, shm, s>>>(p, vals64, out);

@@ -448,7 +448,7 @@ template <typename T, int R, int N>
 cudaError_t run_fused(const FusedParams &p, cudaStream_t s) {
     const size_t shm = fused_smem(N, R, p.warp_floats, p.table_buckets).total;
     auto kern = k_mttkrp_fused<T, R, N>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    cudaError_t e = allow_smem((const void *)kern, shm);
     if (e != cudaSuccess) return e;
     const int grid = grid_for((const void *)kern, shm, p.end - p.begin);
     kern<<<grid, kThreads, shm, s>>>(p);
@@ -461,7 +461,7 @@ cudaError_t run_fused_tiled(const FusedParams &p, cudaStream_t s) {
     const size_t shm = (size_t)(N + 1) * staged<P>() * sizeof(uint32_t) +
                        (size_t)kWarps * (p.warp_floats * sizeof(float) + p.warp_floats / R * sizeof(uint32_t));
     auto kern = k_mttkrp_fused_tiled<T, R, N>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    cudaError_t e = allow_smem((const void *)kern, shm);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, shm) != cudaSuccess || per_sm < 1)

@@ -714,7 +714,7 @@ cudaError_t run_mttkrp_impl(const KParams &p, cudaStream_t s) {
     const int nb = p.log2nb >= 0 ? (1 << p.log2nb) : 0;
     const size_t shm = smem_layout(sizeof(MStage<NG>), p.kw, R, nb).total;
     auto kern = k_mttkrp<T, R, NG, COMP>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    cudaError_t e = allow_smem((const void *)kern, shm);
     if (e != cudaSuccess) return e;
     const int grid = grid_for((const void *)kern, shm, p.end - p.begin);
     kern<<<grid, kThreads, shm, s>>>(p);

@@ -586,10 +586,8 @@ int resident_clusters(K kern, const cudaLaunchConfig_t &cfg, std::atomic<uint64_
 
 template <typename K>
 cudaError_t launch_tiled(K kern, const TParams &p, size_t shm, std::atomic<uint64_t> &last, cudaStream_t s) {
-    if (shm > 48 * 1024) {  // what a kernel may use without asking
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem((const void *)kern, shm);
+    if (e != cudaSuccess) return e;
     const int64_t tiles = (p.nnz + kTile - 1) / kTile;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kTiledCluster);

@@ -235,7 +235,7 @@ cudaError_t build_tile_order(const StoreView &sv, const Layout &L, const HotRows
         a.nhot[n] = std::min(hot[n].count, kOrderCold);
     }
     const size_t shm = (size_t)sv.N * kHotBuckets * sizeof(uint4) + (size_t)kOrderWarps * kTile * 6;
-    cudaError_t e = cudaFuncSetAttribute(k_tile_order, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    cudaError_t e = allow_smem((const void *)k_tile_order, shm);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (sv.end + kTile - 1) / kTile;
     const int64_t grid = std::min<int64_t>((tiles + kOrderWarps - 1) / kOrderWarps, (int64_t)sm_count() * 4);
