@@ -116,9 +116,11 @@ __device__ __forceinline__ void dot2_add(float x, float y, float &hi, float &lo)
 // and CTAs in float64) is off by at most 8e-16, the float64 sum it stands for
 // by 4e-15; Dot2, whose error grows with the terms of a thread, by 5e-13 at 500.
 // All that while the products are in float32's range: one is off by up to
-// 2^-149 where it or its error underflows, which 2^22 terms keep below 2^-53 of
-// a sum of 2^-70 or more, and not finite where it overflows. trusted() tells; a
-// thread whose sum is not takes it again in float64.
+// 2^-149 where it or its error underflows, which 2^23 terms keep below 2^-56 of
+// a sum of 2^-70 or more, and not finite where it overflows. So a CTA (a warp in
+// k_norm2) takes a sum that is not trusted() again in float64. A sum of 0 is
+// trusted where every x is 0 (`seen`: the x's bits ORed is not 0 for any of its
+// threads), as in rows without nonzeros.
 struct WideSum {
     float hi = 0.f, mid = 0.f, lo = 0.f;
     __device__ __forceinline__ void add(const float (&x)[4], const float (&y)[4]) {
@@ -138,11 +140,16 @@ struct WideSum {
         two_sum(mid, a, mid, c);
         lo = __fadd_rn(lo, __fadd_rn(b, c));
     }
-    __device__ __forceinline__ bool trusted() const {
-        return fabsf(hi) >= 0x1p-70f && fabsf(hi) < INFINITY && fabsf(__fadd_rn(mid, lo)) < INFINITY;
-    }
     __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
 };
+
+__device__ __forceinline__ bool trusted(double sum, bool seen) {
+    return (sum == 0.0 && !seen) || (fabs(sum) >= 0x1p-70 && fabs(sum) < INFINITY);
+}
+
+__device__ __forceinline__ uint32_t bits_of(const float (&x)[4]) {
+    return (__float_as_uint(x[0]) | __float_as_uint(x[1]) | __float_as_uint(x[2]) | __float_as_uint(x[3])) & 0x7FFFFFFFu;
+}
 
 // Column scales from the columns' sums of squares: lambda = sqrt, 1 / lambda
 // (1 for a zero column).
@@ -542,6 +549,7 @@ __global__ void __launch_bounds__(kApplyThreads, 4) k_apply(const float *M, int6
     }
     const bool vec = R == sh.R4 && ((reinterpret_cast<uintptr_t>(M) | reinterpret_cast<uintptr_t>(A)) & 15) == 0;
     WideSum sq[4];
+    uint32_t seen = 0;  // of all four columns
     const int64_t ntiles = (I + sh.rows - 1) / sh.rows;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t i0 = t * sh.rows;
@@ -602,34 +610,48 @@ __global__ void __launch_bounds__(kApplyThreads, 4) k_apply(const float *M, int6
         for (int n = 0; n < 4; ++n) {
             const float x[4] = {acc[0][n], acc[1][n], acc[2][n], acc[3][n]};
             sq[n].add(x, x);
+            seen |= bits_of(x);
         }
     }
     __syncthreads();
     double *red = reinterpret_cast<double *>(smem);  // [rg][R4]
     if (rg < sh.rg)
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            red[rg * sh.R4 + c + n] =
-                c + n >= R || sq[n].trusted() ? sq[n].value() : stored_squares(A, I, R, c + n, rg);
-        }
-    __syncthreads();
-    if (tid < R) {
+        for (int n = 0; n < 4; ++n) red[rg * sh.R4 + c + n] = sq[n].value();
+    const bool any = __syncthreads_or(seen != 0);
+    const auto column_sum = [&]() {
         double v = 0.0;
         for (int g = 0; g < sh.rg; ++g) v += red[g * sh.R4 + tid];
-        atomicAdd(&colsq[tid], v);
+        return v;
+    };
+    __shared__ bool again[kSolveMaxRank];
+    double v = 0.0;
+    if (tid < R) {
+        v = column_sum();
+        again[tid] = !trusted(v, any);
     }
+    if (__syncthreads_or(tid < R && again[tid])) {
+        if (rg < sh.rg)
+            for (int n = 0; n < 4 && c + n < R; ++n)
+                if (again[c + n]) red[rg * sh.R4 + c + n] = stored_squares(A, I, R, c + n, rg);
+        __syncthreads();
+        if (tid < R) v = column_sum();
+    }
+    if (tid < R) atomicAdd(&colsq[tid], v);
 }
 
-// <M, A> per column (WideSum, float64 between threads and CTAs) -> acc[R]
-__global__ void __launch_bounds__(256) k_coldot(const float *__restrict__ M, const float *__restrict__ A, int64_t I,
-                                                int R, double *__restrict__ acc) {
+// <M, A> per column (WideSum, float64 between threads and CTAs) -> acc[R]. One
+// round of kColdotCtas CTAs per SM, as many as its registers allow.
+constexpr int kColdotCtas = 6;
+__global__ void __launch_bounds__(256, kColdotCtas) k_coldot(const float *__restrict__ M, const float *__restrict__ A,
+                                                   int64_t I, int R, double *__restrict__ acc) {
     __shared__ double red[256];
     const int nsub = 256 / R;
     const int c = threadIdx.x % R, sub = threadIdx.x / R;
-    double part = 0.0;
+    const int64_t first = (int64_t)blockIdx.x * nsub + sub, step = (int64_t)gridDim.x * nsub;
+    WideSum d;
+    uint32_t seen = 0;
     if (sub < nsub) {
-        const int64_t first = (int64_t)blockIdx.x * nsub + sub, step = (int64_t)gridDim.x * nsub;
-        WideSum d;
         int64_t i = first;
         for (; i + 3 * step < I; i += 4 * step) {
             float x[4], y[4];
@@ -639,24 +661,37 @@ __global__ void __launch_bounds__(256) k_coldot(const float *__restrict__ M, con
                 y[k] = A[(i + k * step) * R + c];
             }
             d.add(x, y);
+            seen |= bits_of(x);
         }
         for (; i < I; i += step) {
             const float x[4] = {M[i * R + c], 0.f, 0.f, 0.f}, y[4] = {A[i * R + c], 0.f, 0.f, 0.f};
             d.add(x, y);
-        }
-        part = d.value();
-        if (!d.trusted()) {
-            part = 0.0;
-            for (int64_t i = first; i < I; i += step) part += (double)M[i * R + c] * (double)A[i * R + c];
+            seen |= bits_of(x);
         }
     }
-    red[threadIdx.x] = part;
-    __syncthreads();
-    if (threadIdx.x < R) {
+    red[threadIdx.x] = d.value();
+    const bool any = __syncthreads_or(seen != 0);
+    const auto column_sum = [&]() {
         double v = 0.0;
         for (int g = 0; g < nsub; ++g) v += red[g * R + threadIdx.x];
-        atomicAdd(&acc[threadIdx.x], v);
+        return v;
+    };
+    __shared__ bool again[128];
+    double v = 0.0;
+    if (threadIdx.x < R) {
+        v = column_sum();
+        again[threadIdx.x] = !trusted(v, any);
     }
+    if (__syncthreads_or(threadIdx.x < R && again[threadIdx.x])) {
+        if (sub < nsub && again[c]) {
+            double part = 0.0;
+            for (int64_t i = first; i < I; i += step) part += (double)M[i * R + c] * (double)A[i * R + c];
+            red[threadIdx.x] = part;
+        }
+        __syncthreads();
+        if (threadIdx.x < R) v = column_sum();
+    }
+    if (threadIdx.x < R) atomicAdd(&acc[threadIdx.x], v);
 }
 
 __global__ void __launch_bounds__(256) k_fit_final(double normX2, const GramPtrs gp, int N, int R,
@@ -696,21 +731,29 @@ __global__ void __launch_bounds__(256) k_fit_final(double normX2, const GramPtrs
 __global__ void __launch_bounds__(256) k_norm2(const float *__restrict__ v, int64_t n, double *__restrict__ out) {
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     WideSum d;
+    uint32_t seen = 0;
     int64_t i = first;
     for (; i + 3 * step < n; i += 4 * step) {
         const float x[4] = {v[i], v[i + step], v[i + 2 * step], v[i + 3 * step]};
         d.add(x, x);
+        seen |= bits_of(x);
     }
     for (; i < n; i += step) {
         const float x[4] = {v[i], 0.f, 0.f, 0.f};
         d.add(x, x);
+        seen |= bits_of(x);
     }
-    double s = d.value();
-    if (!d.trusted()) {
+    const auto warp_sum = [](double s) {
+        for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+        return s;
+    };
+    double s = warp_sum(d.value());
+    const bool any = __any_sync(kFull, seen != 0);
+    if (__any_sync(kFull, !trusted(s, any))) {  // (every lane has the same sum, up to the order of its additions)
         s = 0.0;
-        for (int64_t i = first; i < n; i += step) s += (double)v[i] * (double)v[i];
+        for (i = first; i < n; i += step) s += (double)v[i] * (double)v[i];
+        s = warp_sum(s);
     }
-    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
 }
 
@@ -899,7 +942,10 @@ cudaError_t launch_cpals_fit(double normX2, const double *const *grams, int N, i
     cudaError_t e = cudaMallocAsync(&dots, sizeof(double) * R, s);
     if (e != cudaSuccess) return e;
     k_zero_d<<<1, 128, 0, s>>>(dots, R);
-    if (I > 0) k_coldot<<<grid_cap(I, 256 / R), 256, 0, s>>>(M, A, I, R, dots);
+    if (I > 0) {
+        const int64_t ctas = std::min<int64_t>(grid_cap(I, 256 / R), (int64_t)sm_count() * kColdotCtas);
+        k_coldot<<<(unsigned)ctas, 256, 0, s>>>(M, A, I, R, dots);
+    }
     k_fit_final<<<1, 256, 0, s>>>(normX2, gp, N, R, lambda, dots, fit);
     e = cudaGetLastError();
     cudaFreeAsync(dots, s);

@@ -149,3 +149,18 @@ def test_cp_als_does_not_depend_on_the_units_of_the_values(exponent):
     np.testing.assert_allclose(got[1][1], got[0][1], rtol=tol)
     for a, b in zip(got[0][0], got[1][0]):
         assert np.linalg.norm(a - b) <= tol * np.linalg.norm(a)
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1e-22, 1.0, 1e30])
+def test_sums_over_mostly_empty_rows(scale):
+    """Threads that see nothing but zeros (of either sign) beside threads that do not."""
+    rng = np.random.default_rng(8)
+    Mh = np.zeros((200_003, 10))
+    rows = rng.choice(200_003, 900, replace=False)
+    Mh[rows] = rng.standard_normal((900, 10)) * scale
+    Mh[:, 3] = 0.0
+    Mh[::5] *= -1.0
+    _check_columns(Mh.astype(np.float32), blco.blco_cpals_update)
+    v = Mh[:, 0].astype(np.float32)
+    ref = _squares(v)
+    assert abs(_norm2(v) - ref) <= v.size * EPS * ref
