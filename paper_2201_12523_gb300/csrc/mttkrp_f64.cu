@@ -204,7 +204,8 @@ cudaError_t run_mttkrp64(const KParams &p, const double *vals64, double *out, cu
     auto kern = k_mttkrp64<R, NG>;
     cudaError_t e = allow_smem((const void *)kern, shm);
     if (e != cudaSuccess) return e;
-    const int grid = grid_for((const void *)kern, shm, p.end - p.begin);
+    static std::atomic<uint64_t> last{0};
+    const int grid = grid_for((const void *)kern, shm, p.end - p.begin, last);
     kern<<<grid, kThreads, shm, s>>>(p, vals64, out);
     return cudaGetLastError();
 }

@@ -450,7 +450,8 @@ cudaError_t run_fused(const FusedParams &p, cudaStream_t s) {
     auto kern = k_mttkrp_fused<T, R, N>;
     cudaError_t e = allow_smem((const void *)kern, shm);
     if (e != cudaSuccess) return e;
-    const int grid = grid_for((const void *)kern, shm, p.end - p.begin);
+    static std::atomic<uint64_t> last{0};
+    const int grid = grid_for((const void *)kern, shm, p.end - p.begin, last);
     kern<<<grid, kThreads, shm, s>>>(p);
     return cudaGetLastError();
 }
@@ -463,11 +464,10 @@ cudaError_t run_fused_tiled(const FusedParams &p, cudaStream_t s) {
     auto kern = k_mttkrp_fused_tiled<T, R, N>;
     cudaError_t e = allow_smem((const void *)kern, shm);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, shm) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
+    static std::atomic<uint64_t> last{0};
+    const int64_t grid = (int64_t)sm_count() * ctas_per_sm((const void *)kern, shm, last);
     const int64_t tiles = (p.end + kTile - 1) / kTile;
-    kern<<<(unsigned)std::min<int64_t>((int64_t)sm_count() * per_sm, tiles), kThreads, shm, s>>>(p);
+    kern<<<(unsigned)std::min<int64_t>(grid, tiles), kThreads, shm, s>>>(p);
     return cudaGetLastError();
 }
 

@@ -38,6 +38,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <atomic>
 #include <cstring>
 
 #include "hot_rows.cuh"
@@ -697,10 +698,35 @@ KParams make_params(const StoreView &sv) {
     return p;
 }
 
-int grid_for(const void *kern, size_t shm, int64_t span) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, shm) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
+// query() for the current device and `shm` bytes of shared memory, which costs as
+// much as a launch: each kernel remembers its last answer with both in `last`. 0
+// where there is none.
+template <typename F>
+int remembered(std::atomic<uint64_t> &last, size_t shm, F &&query) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
+    const uint64_t tag = ((uint64_t)(dev & 0xFF) << 24 | (shm & 0xFFFFFF)) << 32;
+    const uint64_t seen = last.load(std::memory_order_relaxed);
+    if ((seen & ~0xFFFFFFFFull) == tag && (uint32_t)seen != 0) return (int)(uint32_t)seen;
+    int n = 0;
+    if (query(&n) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        return 0;
+    }
+    last.store(tag | (uint32_t)n, std::memory_order_relaxed);
+    return n;
+}
+
+// Resident CTAs of a kernel per SM, at least 1.
+int ctas_per_sm(const void *kern, size_t shm, std::atomic<uint64_t> &last) {
+    const int n = remembered(last, shm, [&](int *per_sm) {
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, kThreads, shm);
+    });
+    return n > 0 ? n : 1;
+}
+
+int grid_for(const void *kern, size_t shm, int64_t span, std::atomic<uint64_t> &last) {
+    const int per_sm = ctas_per_sm(kern, shm, last);
     const int64_t tiles = (span + 31) / 32;
     int64_t grid = (int64_t)sm_count() * per_sm;
     const int64_t need = (tiles + kWarps - 1) / kWarps;
@@ -716,7 +742,8 @@ cudaError_t run_mttkrp_impl(const KParams &p, cudaStream_t s) {
     auto kern = k_mttkrp<T, R, NG, COMP>;
     cudaError_t e = allow_smem((const void *)kern, shm);
     if (e != cudaSuccess) return e;
-    const int grid = grid_for((const void *)kern, shm, p.end - p.begin);
+    static std::atomic<uint64_t> last{0};
+    const int grid = grid_for((const void *)kern, shm, p.end - p.begin, last);
     kern<<<grid, kThreads, shm, s>>>(p);
     return cudaGetLastError();
 }
@@ -724,7 +751,8 @@ cudaError_t run_mttkrp_impl(const KParams &p, cudaStream_t s) {
 template <typename T, int R, int NG>
 cudaError_t run_cp_fwd_impl(const KParams &p, cudaStream_t s) {
     auto kern = k_cp_fwd<T, R, NG>;
-    const int grid = grid_for((const void *)kern, 0, p.end - p.begin);
+    static std::atomic<uint64_t> last{0};
+    const int grid = grid_for((const void *)kern, 0, p.end - p.begin, last);
     kern<<<grid, kThreads, 0, s>>>(p);
     return cudaGetLastError();
 }

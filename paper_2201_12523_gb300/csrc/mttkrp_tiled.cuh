@@ -35,7 +35,6 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "mttkrp_kernels.cuh"
 #include "tile_stage.cuh"
@@ -565,23 +564,13 @@ TParams tiled_params(const StoreView &sv, const TileOrder &to, const void *const
 }
 
 // Clusters of a kernel that are resident at once with `shm` bytes of shared
-// memory (a cluster stays inside a GPC, so that is not the SMs' CTAs over the
-// cluster's size). The query costs as much as a launch: each kernel remembers
-// its last answer, with the device and the size it was for.
+// memory, at least 1 (a cluster stays inside a GPC, so that is not the SMs' CTAs
+// over the cluster's size).
 template <typename K>
 int resident_clusters(K kern, const cudaLaunchConfig_t &cfg, std::atomic<uint64_t> &last) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-    const uint64_t tag = ((uint64_t)(dev & 0xFF) << 24 | (cfg.dynamicSmemBytes & 0xFFFFFF)) << 32;
-    const uint64_t seen = last.load(std::memory_order_relaxed);
-    if ((seen & ~0xFFFFFFFFull) == tag && (uint32_t)seen != 0) return (int)(uint32_t)seen;
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
-        cudaGetLastError();
-        return 1;
-    }
-    last.store(tag | (uint32_t)clusters, std::memory_order_relaxed);
-    return clusters;
+    const int n = remembered(last, cfg.dynamicSmemBytes,
+                             [&](int *clusters) { return cudaOccupancyMaxActiveClusters(clusters, kern, &cfg); });
+    return n > 0 ? n : 1;
 }
 
 template <typename K>
