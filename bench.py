@@ -32,7 +32,6 @@ path); the max time over ranks is used.
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import statistics
@@ -58,17 +57,6 @@ CP_MODEL = "cp-planted-3d-200M"
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_HBM_GBS = 6800.0
 FP32_TOL, BF16_TOL = 1e-5, 1e-2
-
-# DRAM traffic of the MTTKRP kernel per launch from one ncu capture
-# (profiles/), valid only for the kernel source it was taken from (sha256, see
-# mttkrp_src_sha): workload -> record.
-TRAFFIC_RECORDS = {
-    "zipf1.1-4d-500M": {"src_sha256": "e6765c8922a7d71eafc404c1d1ce06398280425ae954f857e53e8aeec58b933b",
-                        "bytes_per_launch": 7.223e9},  # mean of modes 0-3, R = 32, float32 factors
-    "zipf1.2-5d-1B": {"src_sha256": "c16df474c0ced002e24fc1c056d4e7cee614803c50b329a74341cd539b008162",
-                      "bytes_per_launch": 28.785e9},  # one-pass all-mode launch, resident store, R = 16
-}
-
 
 def parse_args(argv=None):
     p = argparse.ArgumentParser()
@@ -197,16 +185,29 @@ def hbm_peak():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-def mttkrp_src_sha(onepass: bool = False) -> str:
-    """sha256 over the sources of the MTTKRP kernel of a resident store (the
-    kernel headers and the order of its tiles, with the one-pass kernel's unit
-    where that runs), to tell whether a recorded ncu traffic figure still
-    describes the kernel being timed."""
-    h = hashlib.sha256()
-    for name in ("mttkrp_kernels.cuh", "tile_order.cu", "mttkrp_fused.cu" if onepass else "mttkrp_tiled.cuh"):
-        with open(os.path.join(ROOT, "paper_2201_12523_gb300", "csrc", name), "rb") as f:
-            h.update(f.read())
-    return h.hexdigest()
+def keeps_order(info: dict) -> bool:
+    """Whether a store keeps the order inside its tiles (at least 2 bytes per
+    nonzero and mode beside the 16 of keys, values and positions), which decides
+    the kernels its calls run."""
+    return not info["streamed"] and info["device_bytes"] >= (16 + 2 * info["order"]) * info["nnz"]
+
+
+def mttkrp_kernel(info: dict, R: int, onepass: bool) -> str:
+    """The kernel of an all-mode step with float32 factors on a store."""
+    tiled = keeps_order(info) and (R > 64 or info["nnz"] >= 1 << 20)
+    if onepass:
+        return f"k_mttkrp_fused{'_tiled' if tiled else ''}<float,{R},{info['order']}>"
+    return f"k_mttkrp{'_tiled' if tiled else ''}<float,{R},{info['order'] - 1}>"
+
+
+def streamed_bound(step_ms: float, upload_ms: float, resident_ms: float, link_ms: float) -> str:
+    """What a step on a queue-streamed store is bound by: the uploads where they
+    were under way for nine tenths of it, else the kernels."""
+    if upload_ms >= 0.9 * step_ms:
+        return ("uploads: under way for %.0f of the step's %.0f ms beside the kernels (%.0f ms at the link's measured "
+                "peak; a resident store's step takes %.0f ms)" % (upload_ms, step_ms, link_ms, resident_ms))
+    return ("kernels: the uploads take %.0f of the step's %.0f ms, a resident store's step %.0f ms"
+            % (upload_ms, step_ms, resident_ms))
 
 
 def algorithmic_bytes(spec, R: int, fbytes: int, mode: int, rows=None) -> int:
@@ -480,17 +481,14 @@ def measure_mttkrp(blco, spec, args, ranks, dev, steps, warmup, *, headline, sam
     if onepass:
         b32 = onepass_bytes(spec, R, 4)
         touched_bytes = onepass_bytes(spec, R, 4, touched)
-        kname = f"k_mttkrp_fused_tiled<float,{R},{spec.order}>"
     else:
         b32 = sum(algorithmic_bytes(spec, R, 4, n) for n in range(spec.order)) / spec.order
         touched_bytes = sum(algorithmic_bytes(spec, R, 4, n, touched) for n in range(spec.order)) / spec.order
-        kname = f"k_mttkrp_tiled<float,{R},{spec.order - 1}>"
     ach, kms, kl = kernel_roofline(prof, kind, b32, peak)
-    rec = TRAFFIC_RECORDS.get(spec.name)
-    traffic = rec["bytes_per_launch"] if rec and rec["src_sha256"] == mttkrp_src_sha(onepass) else None
     res["roofline"] = {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
-                       "frac": (ach / peak) if ach else None, "traffic": traffic,
-                       "kernel": kname,
+                       "frac": (ach / peak) if ach else None,
+                       "traffic": None,  # DRAM bytes per launch: no capture of the present kernels at full size
+                       "kernel": mttkrp_kernel((t_res or t).info(), R, onepass),
                        "launch": "one launch per all-mode step (every mode in one pass)" if onepass
                        else "one launch per mode",
                        "peak_source": peak_src + " (burst copy, MEASURED_PEAKS hbm_gbs)",
@@ -539,9 +537,7 @@ def measure_mttkrp(blco, spec, args, ranks, dev, steps, warmup, *, headline, sam
         link_ms = moved / (link * 1e9) * 1e3
         res["host_link"]["resident_ms_per_step"] = ms_r
         res["host_link"]["link_ms_per_step_at_peak"] = link_ms
-        res["host_link"]["bound"] = ("kernels: the all-mode MTTKRP of a resident store takes %.0f ms, longer than "
-                                     "the %.0f ms the host link needs for the store at its measured peak" % (ms_r, link_ms)
-                                     if ms_r > link_ms else "host link")
+        res["host_link"]["bound"] = streamed_bound(res["ms_per_step"], ums / steps, ms_r, link_ms)
         # the same step with the kernel reading the store in host memory
         outs_h = [torch.empty_like(o) for o in outs]
         step_h = make_step(A, t_hr, outs_h)
