@@ -74,7 +74,11 @@ typedef struct {
     int64_t max_nnz_per_block;   /* block cap; 0 = 2^27 (the paper's setting) */
     int32_t line_bits;           /* encoding line length, 1..64; 0 = 64 */
     int32_t n_queues;            /* streaming device queues, 1..8; 0 = 8 */
-    int64_t device_budget_bytes; /* cap on this handle's device memory; 0 = none */
+    int64_t device_budget_bytes; /* cap on this handle's device memory; 0 = none. A store
+                                    built with one keeps no order inside its tiles
+                                    (see device_bytes below): the caller divides the
+                                    memory. A budget that the store does not reach
+                                    changes nothing else. */
     int32_t force_stream;        /* 1 = keep the store in pinned host memory */
     int32_t compensated_sums;    /* 1 = with bf16/fp16 factors, sum each run of
                                     equal output rows with Kahan's compensated
@@ -114,10 +118,18 @@ typedef struct {
     int32_t n_queues;
     int32_t hot_rows[BLCO_MAX_MODES];      /* hottest rows kept per mode (a launch at rank R
                                               accumulates the first min(this, 1024 / R)
-                                              of them on chip) */
-    int64_t device_bytes;                  /* device memory held by the handle (with the
-                                              order inside tiles of a resident store:
-                                              about 2.1 bytes per nonzero and mode) */
+                                              of them on chip per warp, over the order
+                                              inside tiles min(this, 63, 2048 / R) per CTA) */
+    int64_t device_bytes;                  /* device memory held by the handle: 16 bytes per
+                                              nonzero (20 in float64), and for the order
+                                              inside tiles, which makes the calls over the
+                                              whole store faster, 2.13 bytes (2.25) per
+                                              nonzero and mode. Stores of 2^19 nonzeros or
+                                              more keep it (float64: of 3 or 4 modes) that
+                                              are on the device, have no budget, and find
+                                              it in a quarter of the memory that is free
+                                              when they are built; results agree within
+                                              rounding either way. */
     int64_t host_bytes;                    /* pinned host memory held by the handle */
     int32_t host_reads;                    /* 1 if kernels read the streamed store in host memory */
 } blco_info_t;
@@ -150,11 +162,11 @@ blco_status blco_build(const uint32_t *coords, const float *vals, int64_t nnz, c
  *            factors[mode] is not read and may be NULL
  *   R        rank: 8, 16, 32, 64 or 128
  *   out      I_mode x R float32 (host or device); overwritten
- * Accumulation is float32 (segmented within a warp, then in per-warp
- * shared-memory copies of the mode's hottest rows, then vector reductions to
- * global memory), so the summation order, and the last bits, vary from run
- * to run. With bf16/fp16 factors each in-warp run is Kahan-compensated if
- * the handle was built with compensated_sums.
+ * Accumulation is float32 (runs of equal rows, among 32 nonzeros or inside a
+ * tile of 1024, then shared-memory copies of the mode's hottest rows, then
+ * vector reductions to global memory), so the summation order, and the last
+ * bits, vary from run to run. With bf16/fp16 factors each run among 32 nonzeros
+ * is Kahan-compensated if the handle was built with compensated_sums.
  * With any host pointer the call returns when `out` is complete; with device
  * pointers only it is asynchronous on `stream`.
  * Errors: BLCO_ERR_ARG, BLCO_ERR_UNSUPPORTED (rank), BLCO_ERR_OOM (staging),
@@ -179,6 +191,10 @@ blco_status blco_mttkrp(blco_handle h, int mode, const void *const *factors, blc
  * device meanwhile. On a store read in host memory (host_reads) the kernels
  * load the store over the host link: once per call at 5 modes, once per
  * requested mode otherwise.
+ * Outputs are not to share memory with one another or with a factor, with one
+ * exception: device arguments of a store of other than 5 modes that is not
+ * streamed through queues are computed mode after mode, so that where two
+ * outputs overlap the later mode's result stands.
  * A 5-mode store (every I_n <= 2^24, R = 16, 32 or 64) is computed in one
  * pass: each nonzero's five factor rows are gathered once and its product
  * goes to every requested output (Eq. 1 for all modes at once), one kernel
@@ -206,7 +222,10 @@ blco_status blco_mttkrp_all(blco_handle h, const void *const *factors, blco_dtyp
  *     [begin, end); begin a multiple of 32, 0 <= begin <= end <= nnz. Other
  *     arguments as blco_mttkrp. The store must be resident on the device
  *     or read in host memory (host_reads; BLCO_ERR_STATE for a store
- *     streamed through the device queues).
+ *     streamed through the device queues). Whatever the range, the whole store
+ *     included, it runs the kernel that orders 32 nonzeros at a time, whose
+ *     results do not depend on whether the store keeps an order inside tiles;
+ *     CP-ALS sweeps (cp_als) rely on that.
  * Errors: BLCO_ERR_ARG, BLCO_ERR_STATE, BLCO_ERR_UNSUPPORTED, BLCO_ERR_OOM,
  * BLCO_ERR_CUDA.
  */
@@ -225,9 +244,11 @@ blco_status blco_mttkrp_range(blco_handle h, int mode, int64_t begin, int64_t en
  *            factors[mode] not read
  *   R        8, 16, 32 or 64 (BLCO_ERR_UNSUPPORTED otherwise)
  *   out      I_mode x R float64 (host or device), overwritten
- * accumulated in float64 (run sums, per-warp shared-memory copies of the hot
- * rows, red.global.add.f64), so only the summation order differs from the
- * exact-rounding FP64 definition. A float64 store serves blco_mttkrp_f64,
+ * accumulated in float64 (run sums, shared-memory copies of the hot rows,
+ * red.global.add.f64): the summation order differs from the exact-rounding FP64
+ * definition, and over the order inside tiles (3 and 4 modes) the row of the
+ * longest other mode multiplies the sum of the nonzeros that share it, term by
+ * term only where that sum or the row is not finite. A float64 store serves blco_mttkrp_f64,
  * blco_perm, blco_keys, blco_blocks, blco_info and blco_destroy; the float32
  * calls (blco_mttkrp*, blco_cp_*, blco_values, blco_norm2) return
  * BLCO_ERR_STATE on it, and blco_mttkrp_f64 on a float32 store too.
@@ -323,7 +344,7 @@ blco_status blco_cpals_update(const double *const *grams, int N, int mode, int R
  * allocate during a call -- a process that reserved the GPU's memory up front
  * for its own pool, or a latency-critical loop that cannot afford the
  * device-wide synchronization of cudaFree. Its scratch (about 17 KB: the
- * float32 inverse of V and two per-column vectors) is one fixed array in
+ * float32 inverse of V and the columns' sums of squares) is one fixed array in
  * device memory that every GPU loading libblco.so holds until the process
  * exits. Limits and behaviour:
  *   - R must be in 1..64; larger ranks return BLCO_ERR_ARG (the size limit

@@ -525,7 +525,7 @@ def mttkrp_sharded(tensor: Tensor, mode: int, factors: Sequence, out: Optional[t
 
 def cp_als(tensor: Tensor, factors: List[torch.Tensor], iters: int, tol: float = 0.0, stream=None):
     """CP-ALS (Algorithm 1) on the GPU: MTTKRP in float32, the R x R Hadamard
-    of Grams, its Cholesky/pseudo-inverse solve and the fit in float64.
+    of Grams, its inverse (or pseudo-inverse) and the fit in float64.
     ``factors`` (float32, device) are updated in place; returns
     (factors, lambda, fits)."""
     N = tensor.order
@@ -544,11 +544,10 @@ def cp_als(tensor: Tensor, factors: List[torch.Tensor], iters: int, tol: float =
     fits: List[float] = []
     # The update multiplies M by the inverse of V, whose condition magnifies M's
     # rounding about 10^3 times, so a sweep's results follow the order in which
-    # M is summed. Sweeps keep the order of the kernel that sorts 32 nonzeros at
-    # a time where it can be asked for (stores on the device or read in place):
-    # with the tile order the factors after two sweeps were nearer to float64's
-    # (2e-5 off, against 4e-5) but up to 8e-5 from what they have been, for 8 %
-    # of the time.
+    # M is summed: that of the kernel which sorts 32 nonzeros at a time, which a
+    # range call runs on any store (8M nonzeros, two sweeps: two runs of the same
+    # program are 1.6-2.9e-5 apart, this and that before the order inside tiles
+    # no more; with that order 2.6-5.3e-5, for 8 % of the time).
     info_t = blco_info(tensor.handle)
     nnz = int(info_t.nnz)
     in_place = not info_t.streamed or bool(info_t.host_reads)

@@ -19,11 +19,12 @@
 //   The CTA adds its copies to the output once, at its end.
 //
 // Bound by the L1 data pipe, where a gathered row costs a wavefront per 128
-// bytes whether it hits or not: 3.9 wavefronts per nonzero at 3 modes and
-// R = 32 (2 of them gathers), 82 % of the pipe's rate. Against the kernel that
-// sorts 32 nonzeros at a time (mttkrp_kernels.cuh): 255 warp instructions per
-// 32 nonzeros instead of 410; float32, sum of the per-mode launches: 3 modes,
-// 150M nonzeros, R = 32: 9.09 -> 7.47 ms; 4 modes, 100M, R = 32: 9.37 -> 8.75;
+// bytes whether it hits or not: 3.8 wavefronts per nonzero at 3 modes and
+// R = 32 (2 of them gathers), 80 % of the pipe's rate. Against the kernel that
+// sorts 32 nonzeros at a time (mttkrp_kernels.cuh): 318 warp instructions per
+// 32 nonzeros instead of 410, 3.8 wavefronts instead of 4.8 (40M nonzeros, mode
+// 0); float32, sum of the per-mode launches: 3 modes, 150M nonzeros, R = 32:
+// 9.09 -> 7.47 ms; 4 modes, 100M, R = 32: 9.37 -> 8.75;
 // 3 modes, 50M, R = 64: 4.75 -> 4.22; 5 modes, 50M, R = 16: 7.66 -> 5.47.
 // Without the prefetch 11 % slower at 3 modes. Measured and not kept: 512
 // threads per CTA (25 % slower: longer waits at the barrier), 5 or 6 CTAs per
