@@ -128,7 +128,9 @@ typedef struct {
                                               more keep it (float64: of 3 or 4 modes) that
                                               are on the device, have no budget, and find
                                               it in a quarter of the memory that is free
-                                              when they are built; results agree within
+                                              when they are built, for the modes of which
+                                              fewer than 0.98 of a tile's nonzeros have a
+                                              row to themselves; results agree within
                                               rounding either way. */
     int64_t host_bytes;                    /* pinned host memory held by the handle */
     int32_t host_reads;                    /* 1 if kernels read the streamed store in host memory */

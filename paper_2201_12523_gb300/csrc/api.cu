@@ -462,8 +462,14 @@ HotRows hot_for(const blco_tensor *h, int mode, int R) {
     return hr;
 }
 
-// Whether a call at rank R over the whole store uses its order inside tiles.
-bool use_order(const blco_tensor *h, int R) { return h->d_order && (R > 64 || h->nnz >= kTiledMinNnz); }
+// Whether a call for `mode` at rank R over the whole store uses its order inside
+// tiles; mode -1: for all modes in one pass.
+bool use_order(const blco_tensor *h, int R, int mode) {
+    if (!h->d_order || (R <= 64 && h->nnz < kTiledMinNnz)) return false;
+    for (int n = 0; n < h->L.N; ++n)
+        if ((mode < 0 || n == mode) && !h->order.rank[n]) return false;
+    return true;
+}
 
 // The most frequent rows of `mode`, for kernels that choose how many they hold.
 HotRows hot_all(const blco_tensor *h, int mode) {
@@ -510,7 +516,7 @@ blco_status mttkrp_device(blco_tensor *h, int mode, const FactorSet &fs, blco_dt
     cudaError_t e = cudaSuccess;
     if (!zeroed || dst != out) e = timed(h, "zero", s, [&]() { return launch_zero(dst, n * oc.n, s); });
     if (e != cudaSuccess) return cuda_fail(e, "zero output");
-    const bool tiled = use_order(h, R) && range_end < 0 && !(h->compensated && fdt != BLCO_F32);
+    const bool tiled = use_order(h, R, mode) && range_end < 0 && !(h->compensated && fdt != BLCO_F32);
     blco_status st = over_store(
         h, "mttkrp", vals_ext, s,
         [&](const StoreView &sv, cudaStream_t q) {
@@ -607,6 +613,9 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
     float *tv = nullptr;
     blco_status st = BLCO_OK;
     BuildOut bo;
+    const bool may_order = !o.force_stream && h->budget == 0 && tile_order_supported(h->L) && nnz >= kOrderMinNnz &&
+                           (!no_vals || order_pays_f64(N));
+    bool pays[MAXN] = {};
 #define BAIL(status_expr)       \
     do {                        \
         st = (status_expr);     \
@@ -670,7 +679,18 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
             h->hot_count[n] = (int)std::min<int64_t>(h->L.dims[n], warp_tier_capacity(8));
             rows += h->hot_count[n];
         }
-        e = h->dalloc((void **)&h->d_hot[0], sizeof(uint32_t) * rows);
+        // the modes for which the order inside tiles pays, if the store may have
+        // one; read here, where s has nothing else to do, into counts behind the
+        // hot rows
+        rows += rows & 1;
+        e = h->dalloc((void **)&h->d_hot[0], sizeof(uint32_t) * rows + sizeof(unsigned long long) * MAXN);
+        if (e == cudaSuccess && may_order) {
+            unsigned long long ends[MAXN] = {}, *d_ends = reinterpret_cast<unsigned long long *>(h->d_hot[0] + rows);
+            e = sample_run_ends(h->view(), d_ends, s);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(ends, d_ends, sizeof(ends), cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            for (int n = 0; n < N; ++n) pays[n] = order_pays(ends[n], nnz);
+        }
         for (int n = 0; n < N && e == cudaSuccess; ++n) {
             const int64_t I = h->L.dims[n];
             if (n > 0) h->d_hot[n] = h->d_hot[n - 1] + h->hot_count[n - 1];
@@ -759,13 +779,13 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
     // The order inside tiles: for stores without a device budget (which is the
     // caller's to divide) that have it in a quarter of the free memory. A store
     // without it is served by the kernels that order 32 nonzeros at a time.
-    if (!h->streamed && h->budget == 0 && tile_order_supported(h->L) && nnz >= kOrderMinNnz &&
-        (!no_vals || order_pays_f64(N))) {
-        const size_t ob = tile_order_bytes(nnz, N, no_vals);
+    if (may_order) {
+        const size_t ob = tile_order_bytes(nnz, (int)std::count(pays, pays + MAXN, true), no_vals);
         size_t free_b = 0, total_b = 0;
-        if ((ob <= ((size_t)16 << 20) || (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && ob <= free_b / 4)) &&
+        if (ob > 0 &&
+            (ob <= ((size_t)16 << 20) || (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && ob <= free_b / 4)) &&
             h->dalloc(&h->d_order, ob) == cudaSuccess) {
-            h->order = tile_order_view(h->d_order, nnz, N, no_vals);
+            h->order = tile_order_view(h->d_order, nnz, pays, no_vals);
             HotRows hot[MAXN];
             for (int n = 0; n < N; ++n) hot[n] = hot_all(h, n);
             e = build_tile_order(h->view(), h->L, hot, h->order, s);
@@ -909,7 +929,7 @@ blco_status blco_mttkrp_f64(blco_handle h, int mode, const double *const *factor
     if (h->nnz > 0) {
         StoreView sv = h->view();
         e = timed(h, "mttkrp_f64", s, [&]() {
-            if (h->d_order) return launch_mttkrp_tiled_f64(sv, h->order, fs, R, mode, hot_all(h, mode), o, s);
+            if (h->order.rank[mode]) return launch_mttkrp_tiled_f64(sv, h->order, fs, R, mode, hot_all(h, mode), o, s);
             return launch_mttkrp_f64(sv, fs, R, mode, hot, o, s);
         });
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
@@ -1078,7 +1098,7 @@ static blco_status mttkrp_all_onepass(blco_tensor *h, FactorSet fs, const bool *
         if (fused)
             return timed(h, "mttkrp_all_fused", q,
                          [&]() {
-                             return launch_mttkrp_fused(sv, use_order(h, R) ? &h->order : nullptr, fs, fdt, R, hot_all,
+                             return launch_mttkrp_fused(sv, use_order(h, R, -1) ? &h->order : nullptr, fs, fdt, R, hot_all,
                                                         dst_all, q);
                          });
         for (int n = 0; n < N; ++n) {

@@ -69,7 +69,8 @@ struct FactorSet {
     const void *ptr[MAXN];
 };
 
-// The order inside tiles of kTile store positions (tile_order.cu), per mode.
+// The order inside tiles of kTile store positions (tile_order.cu), per mode
+// (NULL: none for this mode).
 struct TileOrder {
     uint16_t *rank[MAXN] = {};   // per store position: rank inside its tile | place of its row among the hottest << 10
     uint32_t *ends[MAXN] = {};   // bit per rank: last nonzero of a run of equal target rows
@@ -124,8 +125,10 @@ cudaError_t launch_mttkrp_fused(const StoreView &sv, const TileOrder *to, const 
 // tile_order.cu
 int order_partner(const int64_t *dims, int N, int mode);
 bool tile_order_supported(const Layout &L);  // at least two modes, of at most 2^31 rows each
-size_t tile_order_bytes(int64_t nnz, int N, bool fibers);
-TileOrder tile_order_view(void *buf, int64_t nnz, int N, bool fibers);
+cudaError_t sample_run_ends(const StoreView &sv, unsigned long long *count, cudaStream_t s);  // of MAXN modes
+bool order_pays(unsigned long long run_ends, int64_t nnz);
+size_t tile_order_bytes(int64_t nnz, int modes, bool fibers);
+TileOrder tile_order_view(void *buf, int64_t nnz, const bool *modes, bool fibers);
 cudaError_t build_tile_order(const StoreView &sv, const Layout &L, const HotRows *hot, const TileOrder &to,
                              cudaStream_t s);
 // mttkrp_tiled_*.cu: the MTTKRP of a whole store with its tile order

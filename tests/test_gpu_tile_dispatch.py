@@ -6,6 +6,10 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
+from tests._util import FP32_TOL
+from tests.test_gpu_tiled import _coo, _i32
+
 pytestmark = pytest.mark.gpu
 
 blco = pytest.importorskip("paper_2201_12523_gb300.blco")
@@ -43,3 +47,38 @@ def test_small_stores_keep_no_order(dtype, dims):
         assert _order_bytes(dims, nnz, dtype) == 0
     for nnz in (1 << 19, (1 << 19) + 1):
         assert _order_bytes(dims, nnz, dtype) == _expected(len(dims), nnz, dtype == torch.float64)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_modes_whose_rows_hardly_repeat_keep_no_order(dtype):
+    """Of 2^20 uniform nonzeros, 1024 neighbours in the store have about 2^16 rows
+    of the long modes to fall on (0.99 of them end a run), and 300 of the short."""
+    nnz = 1 << 20
+    assert _order_bytes((1 << 22, 1 << 21, 300), nnz, dtype) == _expected(1, nnz, dtype == torch.float64)
+    assert _order_bytes((1 << 22, 1 << 21, 1 << 20), nnz, dtype) == 0
+
+
+def test_a_store_with_the_order_of_one_mode_serves_all():
+    dims, nnz, R = (1 << 22, 1 << 21, 300), (1 << 20) + 5, 16
+    rng, c = _coo(dims, nnz, 9, power=1)
+    vals = rng.standard_normal(nnz).astype(np.float32)
+    t = blco.Tensor.build(_i32(c), torch.from_numpy(vals).cuda(), dims)
+    A = [rng.standard_normal((d, R)).astype(np.float32) for d in dims]
+    dA = [torch.from_numpy(a).cuda() for a in A]
+    every = t.mttkrp_all(dA)
+    for n in range(3):
+        M, S = oracle.mttkrp(c, vals.astype(np.float64), dims, [a.astype(np.float64) for a in A], n)
+        assert oracle.max_rel_err(t.mttkrp(n, dA).cpu().numpy(), M, S) <= FP32_TOL
+        assert oracle.max_rel_err(every[n].cpu().numpy(), M, S) <= FP32_TOL
+
+
+def test_one_pass_over_5_modes_without_every_modes_order():
+    dims, nnz, R = (1 << 22, 1 << 20, 40, 30, 20), (1 << 20) + 5, 16
+    rng, c = _coo(dims, nnz, 10, power=1)
+    vals = rng.standard_normal(nnz).astype(np.float32)
+    t = blco.Tensor.build(_i32(c), torch.from_numpy(vals).cuda(), dims)
+    A = [rng.standard_normal((d, R)).astype(np.float32) for d in dims]
+    every = t.mttkrp_all([torch.from_numpy(a).cuda() for a in A])
+    for n in range(5):
+        M, S = oracle.mttkrp(c, vals.astype(np.float64), dims, [a.astype(np.float64) for a in A], n)
+        assert oracle.max_rel_err(every[n].cpu().numpy(), M, S) <= FP32_TOL
