@@ -44,6 +44,12 @@ constexpr int64_t kDefaultCap = (int64_t)1 << 27;
 //   float64, 3 and 4 modes: 70k 0.6-1.0, 200k 0.8-1.3, 500k 0.82-1.46, 1M 1.1-1.5.
 constexpr int64_t kOrderMinNnz = (int64_t)1 << 19;
 constexpr int64_t kTiledMinNnz = (int64_t)1 << 20;
+// Most bytes of outputs that an all-mode call zeroes by one launch before its
+// first mode: half of L2, where they stay until their mode adds to them. Against
+// a launch per mode (3 and 4 modes, 60k / 500k nonzeros): 0.1 MB 34.7 -> 27.0 /
+// 65.7 -> 55.9 us, 49 MB 49.3 -> 41.1 / 117 -> 109, 93 MB 57.4 -> 52.7 / 127.1 ->
+// 127.6, 207 MB 78.7 -> 72.0 / 173 -> 179.
+constexpr int64_t kZeroAtOnce = (int64_t)64 << 20;
 // Modes for which a float64 store keeps it: those k_mttkrp64_tiled is faster at.
 bool order_pays_f64(int N) { return N == 3 || N == 4; }
 
@@ -498,6 +504,11 @@ bool copy_buffer(blco_tensor *h, size_t bytes, float **p) {
     return true;
 }
 
+// Private output copies of a mode at rank R (1: none).
+int copies_of(const blco_tensor *h, int mode, int R) {
+    return hot_for(h, mode, R).dense ? 1 : output_copies(h->L.dims[mode], R);
+}
+
 blco_status mttkrp_device(blco_tensor *h, int mode, const FactorSet &fs, blco_dtype fdt, int R, float *out,
                           const float *vals_ext, cudaStream_t s, int64_t range_begin = 0, int64_t range_end = -1,
                           bool zeroed = false) {
@@ -506,7 +517,7 @@ blco_status mttkrp_device(blco_tensor *h, int mode, const FactorSet &fs, blco_dt
     // short modes: reduce into one private copy per SM, then sum the copies
     OutCopies oc;
     float *dst = out;
-    const int nc = hot.dense ? 1 : output_copies(h->L.dims[mode], R);
+    const int nc = copies_of(h, mode, R);
     if (nc > 1 && copy_buffer(h, sizeof(float) * (size_t)nc * n, &dst)) {
         oc.n = nc;
         oc.stride = n;
@@ -1163,14 +1174,20 @@ blco_status blco_mttkrp_all(blco_handle h, const void *const *factors, blco_dtyp
     if (fused || (h->streamed && !h->host_reads))
         return mttkrp_all_onepass(h, fs, host_in, host_out, in_off, out_off, total, fdt, R, outs, s, fused);
     if (total == 0) {  // device arguments: the modes one after another on s
-        // every output zeroed by one launch, unless one of them shares memory
-        // with a factor that an earlier mode still gathers, or with another
-        // output (of which the later mode's result stands)
-        int64_t len[MAXN] = {};
+        // every output zeroed by one launch (those of modes summed from private
+        // copies need it not), unless one of them shares memory with a factor
+        // that an earlier mode still gathers, or with another output (of which
+        // the later mode's result stands)
+        int64_t len[MAXN] = {}, at_once = 0;
+        float *zero[MAXN] = {};
         bool apart = true;
         for (int n = 0; n < N; ++n) {
             if (!outs[n]) continue;
             len[n] = h->L.dims[n] * (int64_t)R;
+            if (copies_of(h, n, R) == 1) {
+                zero[n] = outs[n];
+                at_once += len[n] * (int64_t)sizeof(float);
+            }
             const uintptr_t o0 = reinterpret_cast<uintptr_t>(outs[n]), o1 = o0 + len[n] * sizeof(float);
             const auto clear_of = [&](const void *a, size_t bytes) {
                 const uintptr_t a0 = reinterpret_cast<uintptr_t>(a);
@@ -1180,13 +1197,14 @@ blco_status blco_mttkrp_all(blco_handle h, const void *const *factors, blco_dtyp
             for (int k = 0; k < n; ++k)
                 if (outs[k]) apart &= clear_of(outs[k], len[k] * sizeof(float));
         }
-        if (apart) {
-            cudaError_t e = timed(h, "zero", s, [&]() { return launch_zero_list(outs, len, N, s); });
+        apart &= at_once <= kZeroAtOnce;
+        if (apart && at_once > 0) {
+            cudaError_t e = timed(h, "zero", s, [&]() { return launch_zero_list(zero, len, N, s); });
             if (e != cudaSuccess) return cuda_fail(e, "zero outputs");
         }
         for (int n = 0; n < N; ++n) {
             if (!outs[n]) continue;
-            st = mttkrp_device(h, n, fs, fdt, R, outs[n], nullptr, s, 0, -1, apart);
+            st = mttkrp_device(h, n, fs, fdt, R, outs[n], nullptr, s, 0, -1, apart && zero[n]);
             if (st != BLCO_OK) return st;
         }
         return BLCO_OK;

@@ -796,29 +796,31 @@ cudaError_t launch_zero(float *p, int64_t n, cudaStream_t s) {
 namespace {
 struct ZeroList {
     float4 *p[MAXN];
-    int64_t n4[MAXN];
+    int64_t end[MAXN];  // of array k among all of them, one after another
+    int count;
 };
 __global__ void k_zero_list(const ZeroList z) {
-    float4 *p = z.p[blockIdx.y];
-    const int64_t n4 = z.n4[blockIdx.y];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int64_t total = z.end[z.count - 1];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        int k = 0;
+        while (i >= z.end[k]) ++k;
+        z.p[k][k > 0 ? i - z.end[k - 1] : i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 }
 }  // namespace
 
 // Zeroes several 16-byte aligned arrays, of multiples of 4 floats, in one launch.
 cudaError_t launch_zero_list(float *const *p, const int64_t *n, int count, cudaStream_t s) {
     ZeroList z = {};
-    int64_t longest = 0;
-    int used = 0;
+    int64_t total = 0;
     for (int i = 0; i < count; ++i) {
         if (!p[i] || n[i] <= 0) continue;
-        z.p[used] = reinterpret_cast<float4 *>(p[i]);
-        z.n4[used++] = n[i] / 4;
-        longest = std::max(longest, n[i] / 4);
+        total += n[i] / 4;
+        z.p[z.count] = reinterpret_cast<float4 *>(p[i]);
+        z.end[z.count++] = total;
     }
-    if (used == 0) return cudaSuccess;
-    k_zero_list<<<dim3(grid_cap(longest, 256), (unsigned)used), 256, 0, s>>>(z);
+    if (z.count == 0) return cudaSuccess;
+    k_zero_list<<<grid_cap(total, 256), 256, 0, s>>>(z);
     return cudaGetLastError();
 }
 
