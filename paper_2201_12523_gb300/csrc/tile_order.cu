@@ -5,7 +5,8 @@
 // hottest rows (6 bits), and one bit per rank for the last nonzero of a run of
 // equal target rows; float64 stores also keep one for the last of a fiber
 // (equal target and partner rows, the partner being the longest other mode).
-// 2.13 bytes per nonzero and mode (2.25 for float64), next to the store's 12.
+// 2.13 bytes per nonzero and mode (2.25 for float64), next to the store's 12,
+// for the modes where order_pays().
 //
 // Why: a kernel that orders 32 nonzeros at a time spends 152 of its 410 warp
 // instructions per 32 nonzeros on that, and ends a run at 0.34-0.65 of the
