@@ -116,11 +116,12 @@ __device__ __forceinline__ void dot2_add(float x, float y, float &hi, float &lo)
 // and CTAs in float64) is off by at most 8e-16, the float64 sum it stands for
 // by 4e-15; Dot2, whose error grows with the terms of a thread, by 5e-13 at 500.
 // All that while the products are in float32's range: one is off by up to
-// 2^-149 where it or its error underflows, which 2^23 terms keep below 2^-56 of
-// a sum of 2^-70 or more, and not finite where it overflows. So a CTA (a warp in
-// k_norm2) takes a sum that is not trusted() again in float64. A sum of 0 is
-// trusted where every x is 0 (`seen`: the x's bits ORed is not 0 for any of its
-// threads), as in rows without nonzeros.
+// 2^-149 where it or its error underflows, and not finite where it overflows. A
+// CTA (a warp in k_norm2) adds its sum to the total and takes it again in float64
+// where it is not finite, or where the total so far is not yet large against
+// such errors of all n terms, n 2^-95, with entries other than 0 among its own:
+// when everything is small, not where only a few CTAs' rows are (sweeps of small
+// tensors with long modes, whose rows are mostly empty, lost 5 % to that).
 struct WideSum {
     float hi = 0.f, mid = 0.f, lo = 0.f;
     __device__ __forceinline__ void add(const float (&x)[4], const float (&y)[4]) {
@@ -143,8 +144,15 @@ struct WideSum {
     __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
 };
 
-__device__ __forceinline__ bool trusted(double sum, bool seen) {
-    return (sum == 0.0 && !seen) || (fabs(sum) >= 0x1p-70 && fabs(sum) < INFINITY);
+// Adds a sum to *total. False where it has to be taken again (see above).
+__device__ __forceinline__ bool add_sum(double *total, double sum, bool seen, double enough) {
+    if (!(fabs(sum) < INFINITY)) return false;
+    if (!seen) return true;  // 0
+    return fabs(atomicAdd(total, sum) + sum) >= enough;
+}
+// Puts the float64 sum in its place.
+__device__ __forceinline__ void replace_sum(double *total, double sum, double by) {
+    atomicAdd(total, fabs(sum) < INFINITY ? by - sum : by);
 }
 
 __device__ __forceinline__ uint32_t bits_of(const float (&x)[4]) {
@@ -628,16 +636,15 @@ __global__ void __launch_bounds__(kApplyThreads, 4) k_apply(const float *M, int6
     double v = 0.0;
     if (tid < R) {
         v = column_sum();
-        again[tid] = !trusted(v, any);
+        again[tid] = !add_sum(&colsq[tid], v, any, (double)I * 0x1p-95);
     }
     if (__syncthreads_or(tid < R && again[tid])) {
         if (rg < sh.rg)
             for (int n = 0; n < 4 && c + n < R; ++n)
                 if (again[c + n]) red[rg * sh.R4 + c + n] = stored_squares(A, I, R, c + n, rg);
         __syncthreads();
-        if (tid < R) v = column_sum();
+        if (tid < R && again[tid]) replace_sum(&colsq[tid], v, column_sum());
     }
-    if (tid < R) atomicAdd(&colsq[tid], v);
 }
 
 // <M, A> per column (WideSum, float64 between threads and CTAs) -> acc[R]. One
@@ -680,7 +687,7 @@ __global__ void __launch_bounds__(256, kColdotCtas) k_coldot(const float *__rest
     double v = 0.0;
     if (threadIdx.x < R) {
         v = column_sum();
-        again[threadIdx.x] = !trusted(v, any);
+        again[threadIdx.x] = !add_sum(&acc[threadIdx.x], v, any, (double)I * 0x1p-95);
     }
     if (__syncthreads_or(threadIdx.x < R && again[threadIdx.x])) {
         if (sub < nsub && again[c]) {
@@ -689,9 +696,8 @@ __global__ void __launch_bounds__(256, kColdotCtas) k_coldot(const float *__rest
             red[threadIdx.x] = part;
         }
         __syncthreads();
-        if (threadIdx.x < R) v = column_sum();
+        if (threadIdx.x < R && again[threadIdx.x]) replace_sum(&acc[threadIdx.x], v, column_sum());
     }
-    if (threadIdx.x < R) atomicAdd(&acc[threadIdx.x], v);
 }
 
 __global__ void __launch_bounds__(256) k_fit_final(double normX2, const GramPtrs gp, int N, int R,
@@ -747,14 +753,17 @@ __global__ void __launch_bounds__(256) k_norm2(const float *__restrict__ v, int6
         for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
         return s;
     };
-    double s = warp_sum(d.value());
+    const bool lead = (threadIdx.x & 31) == 0;
+    const double s = warp_sum(d.value());
     const bool any = __any_sync(kFull, seen != 0);
-    if (__any_sync(kFull, !trusted(s, any))) {  // (every lane has the same sum, up to the order of its additions)
-        s = 0.0;
-        for (i = first; i < n; i += step) s += (double)v[i] * (double)v[i];
-        s = warp_sum(s);
+    bool again = false;
+    if (lead) again = !add_sum(out, s, any, 0x1p-63);  // up to 2^32 values, in batches
+    if (__any_sync(kFull, again)) {
+        double t = 0.0;
+        for (i = first; i < n; i += step) t += (double)v[i] * (double)v[i];
+        t = warp_sum(t);
+        if (lead) replace_sum(out, s, t);
     }
-    if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
 }
 
 // out = sum of the private output copies (n floats each, n % 4 == 0,
