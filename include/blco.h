@@ -125,13 +125,14 @@ typedef struct {
                                               inside tiles, which makes the calls over the
                                               whole store faster, 2.13 bytes (2.25) per
                                               nonzero and mode. Stores of 2^19 nonzeros or
-                                              more keep it (float64: of 3 or 4 modes) that
-                                              are on the device, have no budget, and find
-                                              it in a quarter of the memory that is free
-                                              when they are built, for the modes of which
-                                              fewer than 0.98 of a tile's nonzeros have a
-                                              row to themselves; results agree within
-                                              rounding either way. */
+                                              more keep it (float64: 196,608, of 3 or 4
+                                              modes) that are on the device, have no
+                                              budget, and find it in a quarter of the
+                                              memory that is free when they are built, for
+                                              the modes of which fewer than 0.98 of a
+                                              tile's nonzeros have a row to themselves
+                                              (float64 below 2^20 nonzeros: 0.7); results
+                                              agree within rounding either way. */
     int64_t host_bytes;                    /* pinned host memory held by the handle */
     int32_t host_reads;                    /* 1 if kernels read the streamed store in host memory */
 } blco_info_t;

@@ -41,8 +41,11 @@ constexpr int64_t kDefaultCap = (int64_t)1 << 27;
 //     0.62-0.94, 500k 0.92-1.12, 1.05M 0.94-1.15, 5M 1.0-1.18;
 //   R = 128 (8 rows per launch on chip without the order): 66k 0.36-0.9, 200k
 //     0.73-1.1, 500k 0.76-1.3, from 700k 1.0-1.7;
-//   float64, 3 and 4 modes: 70k 0.6-1.0, 200k 0.8-1.3, 500k 0.82-1.46, 1M 1.1-1.5.
+//   float64, 3 and 4 modes, single modes with less than 0.5 run ends per nonzero
+//     (see order_pays): 100k 1.1-1.2 (0.83 at worst), 150k 1.0 (0.77), 200k 1.14
+//     (0.86), 350k 1.2 (0.94); with more than 0.7: 0.93-1.0 up to 1M.
 constexpr int64_t kOrderMinNnz = (int64_t)1 << 19;
+constexpr int64_t kOrderMinNnz64 = (int64_t)3 << 16;
 constexpr int64_t kTiledMinNnz = (int64_t)1 << 20;
 // Most bytes of outputs that an all-mode call zeroes by one launch before its
 // first mode: half of L2, where they stay until their mode adds to them. Against
@@ -624,8 +627,8 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
     float *tv = nullptr;
     blco_status st = BLCO_OK;
     BuildOut bo;
-    const bool may_order = !o.force_stream && h->budget == 0 && tile_order_supported(h->L) && nnz >= kOrderMinNnz &&
-                           (!no_vals || order_pays_f64(N));
+    const bool may_order = !o.force_stream && h->budget == 0 && tile_order_supported(h->L) &&
+                           (no_vals ? nnz >= kOrderMinNnz64 && order_pays_f64(N) : nnz >= kOrderMinNnz);
     bool pays[MAXN] = {};
 #define BAIL(status_expr)       \
     do {                        \
@@ -700,7 +703,7 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
             e = sample_run_ends(h->view(), d_ends, s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(ends, d_ends, sizeof(ends), cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            for (int n = 0; n < N; ++n) pays[n] = order_pays(ends[n], nnz);
+            for (int n = 0; n < N; ++n) pays[n] = order_pays(ends[n], nnz, no_vals && nnz < kTiledMinNnz ? 0.7 : 0.98);
         }
         for (int n = 0; n < N && e == cudaSuccess; ++n) {
             const int64_t I = h->L.dims[n];

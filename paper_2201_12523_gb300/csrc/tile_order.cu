@@ -278,14 +278,15 @@ cudaError_t sample_run_ends(const StoreView &sv, unsigned long long *count, cuda
 // 2^20 nonzeros, R = 16 / 32 / 64): below 0.3 1.29 / 1.23 / 1.18, 0.7-0.8 1.16 /
 // 1.15 / 1.12, 0.96-0.98 1.12 / 1.12 / 1.07, above 1.00 / 0.96 / 0.99 (0.83 on
 // 30M uniform nonzeros of 2^22 x 3M x 100k): there nothing merges, and the rows
-// gathered in store order share more with their neighbours. The same line for
-// float64 (1.03 / 1.00 / 0.96 above it) and for all modes of a 5-mode store in
-// one pass (0.93 / 0.96 / 0.99), which needs every mode's ranks.
-bool order_pays(unsigned long long run_ends, int64_t nnz) {
+// gathered in store order share more with their neighbours. The same `most` of
+// 0.98 for float64 (1.03 / 1.00 / 0.96 above it) and for all modes of a 5-mode
+// store in one pass (0.93 / 0.96 / 0.99), which needs every mode's ranks; 0.7 in
+// float64 below 2^20 nonzeros (from 200k on 1.0-1.3 below it, 0.93-1.0 above).
+bool order_pays(unsigned long long run_ends, int64_t nnz, double most) {
     const int64_t tiles = nnz / kTile;
     if (tiles == 0) return false;
     const int64_t step = (tiles + kSampleTiles - 1) / kSampleTiles;
-    return (double)run_ends < 0.98 * (double)(tiles / step * kTile);
+    return (double)run_ends < most * (double)(tiles / step * kTile);
 }
 
 cudaError_t build_tile_order(const StoreView &sv, const Layout &L, const HotRows *hot, const TileOrder &to,

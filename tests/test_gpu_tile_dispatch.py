@@ -40,13 +40,22 @@ def test_float64_stores_keep_the_order_for_3_and_4_modes(order, kept):
     assert got == (_expected(order, nnz, True) if kept else 0)
 
 
-@pytest.mark.parametrize("dtype,dims", [(torch.float32, (700, 90)), (torch.float32, (700, 300, 90, 40, 9)),
-                                        (torch.float64, (700, 300, 90))])
-def test_small_stores_keep_no_order(dtype, dims):
-    for nnz in (66_000, (1 << 19) - 1):
+@pytest.mark.parametrize("dtype,dims,least", [
+    (torch.float32, (700, 90), 1 << 19), (torch.float32, (700, 300, 90, 40, 9), 1 << 19),
+    (torch.float64, (700, 300, 90), 3 << 16)])
+def test_small_stores_keep_no_order(dtype, dims, least):
+    for nnz in (66_000, least - 1):
         assert _order_bytes(dims, nnz, dtype) == 0
-    for nnz in (1 << 19, (1 << 19) + 1):
+    for nnz in (least, least + 1):
         assert _order_bytes(dims, nnz, dtype) == _expected(len(dims), nnz, dtype == torch.float64)
+
+
+def test_small_float64_stores_need_longer_runs():
+    """1024 neighbours fall on about 3100 rows of 300k nonzeros (0.85 run ends per
+    nonzero) and 2048 rows of 2^20 (0.79): more than 0.7, less than 0.98."""
+    dims = (20_000, 15_000, 10_000)
+    assert _order_bytes(dims, 300_000, torch.float64) == 0
+    assert _order_bytes(dims, 1 << 20, torch.float64) == _expected(3, 1 << 20, True)
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
