@@ -39,7 +39,7 @@ constexpr int64_t kDefaultCap = (int64_t)1 << 27;
 //   float32 and 16-bit, R <= 64: 66k 0.36-1.07, 200k 0.73-1.0, 500k 0.76-1.3,
 //     1.05M 0.93-1.5, 2M 0.95-1.45, 3M 1.0-2.1; one pass over 5 modes: 66k
 //     0.62-0.94, 500k 0.92-1.12, 1.05M 0.94-1.15, 5M 1.0-1.18;
-//   R = 128 (8 rows per launch on chip without the order): 66k 0.36-0.9, 200k
+//   R = 128 (8 rows per warp on chip without the order): 66k 0.36-0.9, 200k
 //     0.73-1.1, 500k 0.76-1.3, from 700k 1.0-1.7;
 //   float64, 3 and 4 modes, single modes with less than 0.5 run ends per nonzero
 //     (see order_pays): 100k 1.1-1.2 (0.83 at worst), 150k 1.0 (0.77), 200k 1.14

@@ -680,11 +680,12 @@ class Scratch {
         if (bytes > ((size_t)32 << 20) && map_api().ok) {
             CUdeviceptr va = 0;
             size_t len = 0;
-            if (!map_block(bytes, &va, &len)) return cudaErrorMemoryAllocation;
-            *out = reinterpret_cast<T *>(va);
-            mapped_.push_back({va, len});
-            return cudaSuccess;
-        }
+            if (map_block(bytes, &va, &len)) {
+                *out = reinterpret_cast<T *>(va);
+                mapped_.push_back({va, len});
+                return cudaSuccess;
+            }
+        }  // no room: the pool may hold memory that it can reuse
         void *p = nullptr;
         const cudaError_t e = cudaMallocAsync(&p, bytes, s);
         if (e != cudaSuccess) return e;

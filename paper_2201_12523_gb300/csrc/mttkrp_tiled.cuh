@@ -20,8 +20,8 @@
 //
 // Bound by the L1 data pipe, where a gathered row costs a wavefront per 128
 // bytes whether it hits or not: 3.8 wavefronts per nonzero at 3 modes and
-// R = 32 (2 of them gathers), 80 % of the pipe's rate. Against the kernel that
-// sorts 32 nonzeros at a time (mttkrp_kernels.cuh): 318 warp instructions per
+// R = 32 (2 of them gathers), 73 % of the pipe's rate. Against the kernel that
+// sorts 32 nonzeros at a time (mttkrp_kernels.cuh): 328 warp instructions per
 // 32 nonzeros instead of 410, 3.8 wavefronts instead of 4.8 (40M nonzeros, mode
 // 0); float32, sum of the per-mode launches: 3 modes, 150M nonzeros, R = 32:
 // 9.09 -> 7.47 ms; 4 modes, 100M, R = 32: 9.37 -> 8.75;
