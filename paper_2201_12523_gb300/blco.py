@@ -545,9 +545,9 @@ def cp_als(tensor: Tensor, factors: List[torch.Tensor], iters: int, tol: float =
     # The update multiplies M by the inverse of V, whose condition magnifies M's
     # rounding about 10^3 times, so a sweep's results follow the order in which
     # M is summed: that of the kernel which sorts 32 nonzeros at a time, which a
-    # range call runs on any store (8M nonzeros, two sweeps: two runs of the same
-    # program are 1.6-2.9e-5 apart, this and that before the order inside tiles
-    # no more; with that order 2.6-5.3e-5, for 8 % of the time).
+    # range call runs on any store (8M nonzeros, two sweeps: two runs of this
+    # program are 1.6-2.9e-5 apart; over the order inside tiles the factors would
+    # be 2.6-5.3e-5 from these, for 8 % less time).
     info_t = blco_info(tensor.handle)
     nnz = int(info_t.nnz)
     in_place = not info_t.streamed or bool(info_t.host_reads)
