@@ -194,7 +194,7 @@ def keeps_order(info: dict) -> bool:
 
 def mttkrp_kernel(info: dict, R: int, onepass: bool) -> str:
     """The kernel of an all-mode step with float32 factors on a store."""
-    tiled = keeps_order(info) and (R > 64 or info["nnz"] >= 1 << 20)
+    tiled = keeps_order(info) and (not 16 <= R <= 64 or info["nnz"] >= 1 << 20)
     if onepass:
         return f"k_mttkrp_fused{'_tiled' if tiled else ''}<float,{R},{info['order']}>"
     return f"k_mttkrp{'_tiled' if tiled else ''}<float,{R},{info['order'] - 1}>"

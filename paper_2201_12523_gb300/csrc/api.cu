@@ -32,17 +32,18 @@ namespace {
 
 constexpr int64_t kDefaultCap = (int64_t)1 << 27;
 // Fewest nonzeros for which the order inside tiles is kept, and from which calls
-// at R <= 64 use it. A launch has a CTA per tile of 1024: below two rounds of
+// at R = 16, 32 and 64 use it. A launch has a CTA per tile of 1024: below two rounds of
 // them over the SMs (1.2M nonzeros at 4 CTAs per SM) the kernels that order 32
 // nonzeros at a time spread the work better. Speed with the order over without,
 // sums over modes of random shapes of 2 to 8 modes, uniform and Zipf:
 //   float32 and 16-bit, R <= 64: 66k 0.36-1.07, 200k 0.73-1.0, 500k 0.76-1.3,
 //     1.05M 0.93-1.5, 2M 0.95-1.45, 3M 1.0-2.1; one pass over 5 modes: 66k
 //     0.62-0.94, 500k 0.92-1.12, 1.05M 0.94-1.15, 5M 1.0-1.18;
+//   R = 8 alone: 300k 0.91-1.07, 500k 1.0-1.27, 700k 0.84-1.07, 850k 0.96-1.37;
 //   R = 128 (8 rows per warp on chip without the order): 66k 0.36-0.9, 200k
 //     0.73-1.1, 500k 0.76-1.3, from 700k 1.0-1.7;
 //   float64, 3 and 4 modes, single modes with less than 0.5 run ends per nonzero
-//     (see order_pays): 100k 1.1-1.2 (0.83 at worst), 150k 1.0 (0.77), 200k 1.14
+//     (run_end_share): 100k 1.1-1.2 (0.83 at worst), 150k 1.0 (0.77), 200k 1.14
 //     (0.86), 350k 1.2 (0.94); with more than 0.7: 0.93-1.0 up to 1M.
 constexpr int64_t kOrderMinNnz = (int64_t)1 << 19;
 constexpr int64_t kOrderMinNnz64 = (int64_t)3 << 16;
@@ -137,6 +138,7 @@ struct blco_tensor {
     // order inside tiles (resident stores; NULL: none)
     void *d_order = nullptr;
     TileOrder order;
+    float run_ends[MAXN] = {};  // run ends per nonzero in a sample of tiles
     // streaming queues
     int64_t queue_nnz = 0;
     uint64_t *q_keys[8] = {};
@@ -474,7 +476,7 @@ HotRows hot_for(const blco_tensor *h, int mode, int R) {
 // Whether a call for `mode` at rank R over the whole store uses its order inside
 // tiles; mode -1: for all modes in one pass.
 bool use_order(const blco_tensor *h, int R, int mode) {
-    if (!h->d_order || (R <= 64 && h->nnz < kTiledMinNnz)) return false;
+    if (!h->d_order || (R >= 16 && R <= 64 && h->nnz < kTiledMinNnz)) return false;
     for (int n = 0; n < h->L.N; ++n)
         if ((mode < 0 || n == mode) && !h->order.rank[n]) return false;
     return true;
@@ -703,7 +705,10 @@ static blco_status build_impl(const uint32_t *coords, const float *vals, int64_t
             e = sample_run_ends(h->view(), d_ends, s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(ends, d_ends, sizeof(ends), cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            for (int n = 0; n < N; ++n) pays[n] = order_pays(ends[n], nnz, no_vals && nnz < kTiledMinNnz ? 0.7 : 0.98);
+            for (int n = 0; n < N; ++n) {
+                h->run_ends[n] = run_end_share(ends[n], nnz);
+                pays[n] = h->run_ends[n] < (no_vals && nnz < kTiledMinNnz ? 0.7f : 0.98f);
+            }
         }
         for (int n = 0; n < N && e == cudaSuccess; ++n) {
             const int64_t I = h->L.dims[n];
@@ -943,7 +948,11 @@ blco_status blco_mttkrp_f64(blco_handle h, int mode, const double *const *factor
     if (h->nnz > 0) {
         StoreView sv = h->view();
         e = timed(h, "mttkrp_f64", s, [&]() {
-            if (h->order.rank[mode]) return launch_mttkrp_tiled_f64(sv, h->order, fs, R, mode, hot_all(h, mode), o, s);
+            // at R = 64 a fiber's end costs two multiply-adds per lane: 1.04 times
+            // the speed without the order at 0.7-0.8 run ends per nonzero, 1.01
+            // (0.98 at worst) at 0.85-0.9, 0.98 at 0.9-0.95, 0.97 above
+            if (h->order.rank[mode] && !(R == 64 && h->run_ends[mode] >= 0.85f))
+                return launch_mttkrp_tiled_f64(sv, h->order, fs, R, mode, hot_all(h, mode), o, s);
             return launch_mttkrp_f64(sv, fs, R, mode, hot, o, s);
         });
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch");

@@ -126,7 +126,7 @@ cudaError_t launch_mttkrp_fused(const StoreView &sv, const TileOrder *to, const 
 int order_partner(const int64_t *dims, int N, int mode);
 bool tile_order_supported(const Layout &L);  // at least two modes, of at most 2^31 rows each
 cudaError_t sample_run_ends(const StoreView &sv, unsigned long long *count, cudaStream_t s);  // of MAXN modes
-bool order_pays(unsigned long long run_ends, int64_t nnz, double most);
+float run_end_share(unsigned long long run_ends, int64_t nnz);
 size_t tile_order_bytes(int64_t nnz, int modes, bool fibers);
 TileOrder tile_order_view(void *buf, int64_t nnz, const bool *modes, bool fibers);
 cudaError_t build_tile_order(const StoreView &sv, const Layout &L, const HotRows *hot, const TileOrder &to,

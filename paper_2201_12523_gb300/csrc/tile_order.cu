@@ -6,7 +6,7 @@
 // equal target rows; float64 stores also keep one for the last of a fiber
 // (equal target and partner rows, the partner being the longest other mode).
 // 2.13 bytes per nonzero and mode (2.25 for float64), next to the store's 12,
-// for the modes where order_pays().
+// for the modes where run_end_share() is low.
 //
 // Why: a kernel that orders 32 nonzeros at a time spends 152 of its 410 warp
 // instructions per 32 nonzeros on that, and ends a run at 0.34-0.65 of the
@@ -262,7 +262,7 @@ TileOrder tile_order_view(void *buf, int64_t nnz, const bool *modes, bool fibers
     return to;
 }
 
-// Run ends per mode in at most kSampleTiles whole tiles, for order_pays().
+// Run ends per mode in at most kSampleTiles whole tiles, for run_end_share().
 cudaError_t sample_run_ends(const StoreView &sv, unsigned long long *count, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned long long) * MAXN, s);
     const int64_t tiles = sv.end / kTile;
@@ -272,21 +272,22 @@ cudaError_t sample_run_ends(const StoreView &sv, unsigned long long *count, cuda
     return cudaGetLastError();
 }
 
-// Whether a mode's runs in tiles are long enough for the order to pay. Speed of
-// the tiled kernels over those that order 32 nonzeros at a time by the share of
-// nonzeros that end a run (random shapes of 2 to 8 modes, uniform and Zipf, from
-// 2^20 nonzeros, R = 16 / 32 / 64): below 0.3 1.29 / 1.23 / 1.18, 0.7-0.8 1.16 /
-// 1.15 / 1.12, 0.96-0.98 1.12 / 1.12 / 1.07, above 1.00 / 0.96 / 0.99 (0.83 on
-// 30M uniform nonzeros of 2^22 x 3M x 100k): there nothing merges, and the rows
-// gathered in store order share more with their neighbours. The same `most` of
-// 0.98 for float64 (1.03 / 1.00 / 0.96 above it) and for all modes of a 5-mode
-// store in one pass (0.93 / 0.96 / 0.99), which needs every mode's ranks; 0.7 in
-// float64 below 2^20 nonzeros (from 200k on 1.0-1.3 below it, 0.93-1.0 above).
-bool order_pays(unsigned long long run_ends, int64_t nnz, double most) {
+// Run ends per nonzero in the sample: whether a mode's runs in tiles are long
+// enough for the order to pay. Speed of the tiled kernels over those that order 32
+// nonzeros at a time by that share (random shapes of 2 to 8 modes, uniform and
+// Zipf, from 2^20 nonzeros, R = 16 / 32 / 64): below 0.3 1.29 / 1.23 / 1.18,
+// 0.7-0.8 1.16 / 1.15 / 1.12, 0.96-0.98 1.12 / 1.12 / 1.07, above 1.00 / 0.96 /
+// 0.99 (0.83 on 30M uniform nonzeros of 2^22 x 3M x 100k): there nothing merges,
+// and the rows gathered in store order share more with their neighbours. So the
+// order is kept below 0.98; the same in float64 (1.03 / 1.00 / 0.96 above it) and
+// for all modes of a 5-mode store in one pass (0.93 / 0.96 / 0.99), which needs
+// every mode's ranks. Float64 below 2^20 nonzeros: 0.7 (from 200k on 1.0-1.3 below
+// it, 0.93-1.0 above).
+float run_end_share(unsigned long long run_ends, int64_t nnz) {
     const int64_t tiles = nnz / kTile;
-    if (tiles == 0) return false;
+    if (tiles == 0) return 1.f;
     const int64_t step = (tiles + kSampleTiles - 1) / kSampleTiles;
-    return (double)run_ends < most * (double)(tiles / step * kTile);
+    return (float)((double)run_ends / (double)(tiles / step * kTile));
 }
 
 cudaError_t build_tile_order(const StoreView &sv, const Layout &L, const HotRows *hot, const TileOrder &to,

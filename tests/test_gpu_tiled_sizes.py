@@ -1,6 +1,6 @@
 """The kernels over the order inside tiles of 1024 positions at the edges of their
 tiles, ranks, gather counts and row widths, on stores large enough to use them
-(2^20 nonzeros; 2^19 at R = 128 and in float64), against the FP64 oracle and
+(2^20 nonzeros; 2^19 at R = 8 and 128 and in float64), against the FP64 oracle and
 against the kernel that orders 32 nonzeros at a time (blco_mttkrp_range).
 Tolerances: float32 sums as everywhere else, float64 sums 1e-12."""
 
@@ -29,6 +29,7 @@ M, H = 1 << 20, 1 << 19
     ((90, 80, 70, 6, 5, 4), M + 4469, 64, 8, torch.float32),           # generic gather count
     ((90, 80, 70, 6, 5, 4, 3, 2), H + 4470, 64, 128, torch.float32),
     ((500, 400, 30), H + 1, 64, 128, torch.bfloat16),
+    ((500, 400, 30), H + 5, 64, 8, torch.float32),
     (((1 << 23) + 5, 1 << 14, 900), M + 4471, 40, 32, torch.float32),  # a row does not fit 22 bits; blocks
     ((1000, 1, 900), M + 4472, 64, 32, torch.float32),                 # a mode of one row
 ])
@@ -37,7 +38,8 @@ def test_mttkrp(dims, nnz, line, R, dtype):
 
 
 @pytest.mark.parametrize("R", [8, 16, 32, 64])
-@pytest.mark.parametrize("dims,nnz", [((500, 400, 30), H), ((200, 90, 30, 7), H + 1), ((4000, 1, 3000), H + 1023)])
+@pytest.mark.parametrize("dims,nnz", [((500, 400, 30), H), ((200, 90, 30, 7), H + 1), ((4000, 1, 3000), H + 1023),
+                                      ((40_000, 30_000, 2000), M + 7)])  # modes with 0.85 run ends per nonzero and more
 def test_mttkrp_f64(dims, nnz, R):
     rng, c = tiled._coo(dims, nnz, R)
     vals = rng.standard_normal(nnz)
